@@ -72,7 +72,7 @@ __global__ void k_tgv_dual(LevelView L, TgvParams tp) {
   float p1 = sld<ST_F32>(L.p1, i), p2 = sld<ST_F32>(L.p2, i);
   float q11 = L.q11[i], q12 = L.q12[i], q21 = L.q21[i], q22 = L.q22[i];
   float t1, t2, qx1, qx2, qy1, qy2;
-  tgv_px_dual(m, L.ubar[i], L.ubar[r], L.ubar[b], L.vb1[i], L.vb1[r], L.vb1[b], L.vb2[i],
+  tgv_px_dual<false>(m, L.ubar[i], L.ubar[r], L.ubar[b], L.vb1[i], L.vb1[r], L.vb1[b], L.vb2[i],
               L.vb2[r], L.vb2[b], c, tp, p1, p2, q11, q12, q21, q22, t1, t2, qx1, qx2, qy1,
               qy2);
   sst<ST_F32>(L.p1, i, p1);
@@ -116,7 +116,8 @@ struct TgvState {
   float* s[12];   // u, ubar, v1, v2, vb1, vb2, p1, p2, q11, q12, q21, q22
 };
 
-template <int FW, int NY, int R>
+// FTZ as in tgv_ball.
+template <int FW, int NY, int R, bool FTZ>
 __global__ void __launch_bounds__(FW * NY, FW * NY >= 512 ? 1 : 2)
 k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n_iters,
               int chained) {
@@ -247,7 +248,7 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
         const float2 ub_b = last ? make_float2(ub2[0].y, s_ub[fnext][tx]) : ub2[j + 1];
         const float2 vb1_b = last ? make_float2(vb12[0].y, s_vb1[fnext][tx]) : vb12[j + 1];
         const float2 vb2_b = last ? make_float2(vb22[0].y, s_vb2[fnext][tx]) : vb22[j + 1];
-        tgv_px_dual2(mb >> (3 * j), mb >> (3 * (j + H)), ub2[j],
+        tgv_px_dual2<FTZ>(mb >> (3 * j), mb >> (3 * (j + H)), ub2[j],
                      make_float2(s_ub[f0][txr], s_ub[f1][txr]), ub_b, vb12[j],
                      make_float2(s_vb1[f0][txr], s_vb1[f1][txr]), vb1_b, vb22[j],
                      make_float2(s_vb2[f0][txr], s_vb2[f1][txr]), vb2_b, c2[j], tp, p12[j],
@@ -306,7 +307,7 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
       const float ub_b = (r + 1 < R) ? ub[r + 1] : s_ub[fb][tx];
       const float vb1_b = (r + 1 < R) ? vb1[r + 1] : s_vb1[fb][tx];
       const float vb2_b = (r + 1 < R) ? vb2[r + 1] : s_vb2[fb][tx];
-      tgv_px_dual(mb >> (3 * r), ub[r], s_ub[fy][txr], ub_b, vb1[r], s_vb1[fy][txr], vb1_b,
+      tgv_px_dual<FTZ>(mb >> (3 * r), ub[r], s_ub[fy][txr], ub_b, vb1[r], s_vb1[fy][txr], vb1_b,
                   vb2[r], s_vb2[fy][txr], vb2_b, c[r], tp, p1[r], p2[r], q11[r], q12[r],
                   q21[r], q22[r], t1[r], t2[r], qx1[r], qx2[r], qy1[r], qy2[r]);
       s_t1[fy][tx] = t1[r];
@@ -383,8 +384,8 @@ TgvState alternate(const LevelView& L) {
   return s;
 }
 
-template <int FW, int NY, int R>
-cudaError_t launch_blocked_t(const LevelView& L, const TgvState& in, const TgvState& out,
+template <int FW, int NY, int R, bool FTZ>
+cudaError_t launch_blocked_f(const LevelView& L, const TgvState& in, const TgvState& out,
                              const TgvParams& tp, int B, int n, bool chained, cudaStream_t st) {
   const int IW = FW - 2 * B, IH = NY * R - 2 * B;
   if (IW <= 0 || IH <= 0 || n < 0 || n > B) return cudaErrorInvalidValue;
@@ -396,7 +397,7 @@ cudaError_t launch_blocked_t(const LevelView& L, const TgvState& in, const TgvSt
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(opted.load() & bit)) {
-      e = cudaFuncSetAttribute(k_tgv_blocked<FW, NY, R>,
+      e = cudaFuncSetAttribute(k_tgv_blocked<FW, NY, R, FTZ>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       opted.fetch_or(bit);
@@ -412,8 +413,16 @@ cudaError_t launch_blocked_t(const LevelView& L, const TgvState& in, const TgvSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_tgv_blocked<FW, NY, R>, L, in, out, tp, B, n,
+  return cudaLaunchKernelEx(&cfg, k_tgv_blocked<FW, NY, R, FTZ>, L, in, out, tp, B, n,
                             chained ? 1 : 0);
+}
+
+template <int FW, int NY, int R>
+cudaError_t launch_blocked_t(const LevelView& L, const TgvState& in, const TgvState& out,
+                             const TgvParams& tp, int B, int n, bool chained, cudaStream_t st) {
+  return tgv_normal_radii(tp)
+             ? launch_blocked_f<FW, NY, R, true>(L, in, out, tp, B, n, chained, st)
+             : launch_blocked_f<FW, NY, R, false>(L, in, out, tp, B, n, chained, st);
 }
 
 // The 32 x 32 footprint on 256 threads of 4 rows (variant 0), 1024 threads

@@ -75,6 +75,18 @@ __device__ __forceinline__ void px_zero(PxConst& c) {
   c.sd = c.tau = c.step = c.c0 = 0.f;
 }
 
+// min(1, 1 / sqrt(n2)) for n2 >= 0 (or NaN).  The .ftz form of the
+// approximate reciprocal square root needs no scaling steps for subnormal
+// inputs; it gives the bits of rsqrtf on normal inputs, and on subnormal
+// ones both are above 1 (checked over all 2^31 non-negative floats).  It
+// takes 4-5 % off an iteration: 100 iterations at 1024 x 1024 (64 x 64
+// footprints of 1024 threads, depth 7) went from 438 to 419 us.
+__device__ __forceinline__ float ball_scale(float n2) {
+  float s;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(n2));
+  return fminf(1.f, s);
+}
+
 // Dual ascent at one pixel: ub, right = ubar(x + e1), below = ubar(x + e2).
 // Updates p1, p2 and returns the masked products t1, t2 of T^1/2 p.
 // MASKED = false is for pixels whose mask bits are all set (in the FOV, both
@@ -92,7 +104,7 @@ __device__ __forceinline__ void px_dual(unsigned m, float ub, float right, float
   float q1 = fmaf(c.sd, k1, __fmul_rn(p1, c.dinv));
   float q2 = fmaf(c.sd, k2, __fmul_rn(p2, c.dinv));
   // P(q) = q / max(1, |q|): scale by min(1, 1/|q|) (1 for |q| <= 1, also q = 0)
-  const float s = fminf(1.f, rsqrtf(fmaf(q1, q1, __fmul_rn(q2, q2))));
+  const float s = ball_scale(fmaf(q1, q1, __fmul_rn(q2, q2)));
   q1 = __fmul_rn(q1, s);
   q2 = __fmul_rn(q2, s);
   p1 = q1;
@@ -175,7 +187,7 @@ __device__ __forceinline__ void px_dual2(unsigned m0, unsigned m1, float2 ub, fl
   float2 q1 = __ffma2_rn(c.sd, k1, __fmul2_rn(p1, c.dinv));
   float2 q2 = __ffma2_rn(c.sd, k2, __fmul2_rn(p2, c.dinv));
   const float2 n2 = __ffma2_rn(q1, q1, __fmul2_rn(q2, q2));
-  const float2 s = make_float2(fminf(1.f, rsqrtf(n2.x)), fminf(1.f, rsqrtf(n2.y)));
+  const float2 s = make_float2(ball_scale(n2.x), ball_scale(n2.y));
   q1 = __fmul2_rn(q1, s);
   q2 = __fmul2_rn(q2, s);
   p1 = q1;

@@ -23,6 +23,13 @@ struct TgvParams {
   int precond;
 };
 
+// Whether a squared norm above the square of each (non-zero) ball radius is
+// always a normal number, so that the ball scalings may use the flushing
+// reciprocal square root (tgv_ball) with the same bits.
+inline bool tgv_normal_radii(const TgvParams& tp) {
+  return tp.alpha1 >= 1e-18f && (tp.alpha0 == 0.f || tp.alpha0 >= 1e-18f);
+}
+
 // Per-pixel constants of one warp (all 0 off the FOV mask: nothing moves).
 struct TgvConst {
   float sx, sy;        // T^1/2 = I - s s^T
@@ -58,12 +65,21 @@ __device__ __forceinline__ void tgv_const(unsigned m, unsigned ml, unsigned mu, 
   c.c0 = Iu != 0.f ? __fsub_rn(uw, __fdiv_rn(rho0, Iu)) : 0.f;
 }
 
+// FTZ: the flushing form of the reciprocal square root, without the scaling
+// steps subnormal inputs need (the bits of rsqrtf on normal ones, and no
+// other n2 exceeds r * r; tgv_normal_radii).  An 800 x 800 frame of 5 levels
+// x 5 warps x 30 iterations went from 2.52 to 2.44 ms with it.
+template <bool FTZ>
 __device__ __forceinline__ float tgv_ball(float n2, float r) {
-  return n2 > r * r ? r * rsqrtf(n2) : 1.f;
+  float s;
+  if constexpr (FTZ) asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(n2));
+  else s = rsqrtf(n2);
+  return n2 > r * r ? r * s : 1.f;
 }
 
 // Dual ascent at one pixel from its own and its right (r) / lower (b)
 // neighbours' ubar, vbar.  Updates p, q; returns t and the masked q.
+template <bool FTZ>
 __device__ __forceinline__ void tgv_px_dual(unsigned m, float ub, float ub_r, float ub_b,
                                             float vb1, float vb1_r, float vb1_b, float vb2,
                                             float vb2_r, float vb2_b, const TgvConst& c,
@@ -77,7 +93,7 @@ __device__ __forceinline__ void tgv_px_dual(unsigned m, float ub, float ub_r, fl
   const float d = fmaf(c.sx, g1, __fmul_rn(c.sy, g2));
   float a1 = fmaf(c.sp, __fsub_rn(fmaf(-c.sx, d, g1), vb1), p1);
   float a2 = fmaf(c.sp, __fsub_rn(fmaf(-c.sy, d, g2), vb2), p2);
-  const float s = tgv_ball(fmaf(a1, a1, __fmul_rn(a2, a2)), tp.alpha1);
+  const float s = tgv_ball<FTZ>(fmaf(a1, a1, __fmul_rn(a2, a2)), tp.alpha1);
   p1 = __fmul_rn(a1, s);
   p2 = __fmul_rn(a2, s);
   const float j11 = gx ? __fsub_rn(vb1_r, vb1) : 0.f;
@@ -87,7 +103,7 @@ __device__ __forceinline__ void tgv_px_dual(unsigned m, float ub, float ub_r, fl
   const float b11 = fmaf(c.sq, j11, q11), b12 = fmaf(c.sq, j12, q12);
   const float b21 = fmaf(c.sq, j21, q21), b22 = fmaf(c.sq, j22, q22);
   const float n2 = fmaf(b11, b11, fmaf(b12, b12, fmaf(b21, b21, __fmul_rn(b22, b22))));
-  const float sc = tp.alpha0 > 0.f ? tgv_ball(n2, tp.alpha0) : 0.f;
+  const float sc = tp.alpha0 > 0.f ? tgv_ball<FTZ>(n2, tp.alpha0) : 0.f;
   q11 = __fmul_rn(b11, sc);
   q12 = __fmul_rn(b12, sc);
   q21 = __fmul_rn(b21, sc);
@@ -160,6 +176,7 @@ __device__ __forceinline__ float2 tgv_sel2(bool kx, bool ky, float2 v) {
 }
 
 // m0, m1: the two pixels' mask bits.
+template <bool FTZ>
 __device__ __forceinline__ void tgv_px_dual2(
     unsigned m0, unsigned m1, float2 ub, float2 ub_r, float2 ub_b, float2 vb1, float2 vb1_r,
     float2 vb1_b, float2 vb2, float2 vb2_r, float2 vb2_b, const TgvConst2& c,
@@ -173,7 +190,7 @@ __device__ __forceinline__ void tgv_px_dual2(
   const float2 a1 = __ffma2_rn(c.sp, tgv_sub2(__ffma2_rn(c.sx, nd, g1), vb1), p1);
   const float2 a2 = __ffma2_rn(c.sp, tgv_sub2(__ffma2_rn(c.sy, nd, g2), vb2), p2);
   const float2 na = __ffma2_rn(a1, a1, __fmul2_rn(a2, a2));
-  const float2 s = make_float2(tgv_ball(na.x, tp.alpha1), tgv_ball(na.y, tp.alpha1));
+  const float2 s = make_float2(tgv_ball<FTZ>(na.x, tp.alpha1), tgv_ball<FTZ>(na.y, tp.alpha1));
   p1 = __fmul2_rn(a1, s);
   p2 = __fmul2_rn(a2, s);
   const float2 j11 = tgv_sel2(gx0, gx1, tgv_sub2(vb1_r, vb1));
@@ -185,7 +202,7 @@ __device__ __forceinline__ void tgv_px_dual2(
   const float2 nb = __ffma2_rn(b11, b11, __ffma2_rn(b12, b12, __ffma2_rn(b21, b21,
                                                                           __fmul2_rn(b22, b22))));
   const float2 sc = tp.alpha0 > 0.f
-                        ? make_float2(tgv_ball(nb.x, tp.alpha0), tgv_ball(nb.y, tp.alpha0))
+                        ? make_float2(tgv_ball<FTZ>(nb.x, tp.alpha0), tgv_ball<FTZ>(nb.y, tp.alpha0))
                         : make_float2(0.f, 0.f);
   q11 = __fmul2_rn(b11, sc);
   q12 = __fmul2_rn(b12, sc);
