@@ -334,7 +334,12 @@ fs_status upload_masks(fs_handle* h, std::vector<uint8_t>& host) {
         if (m && y + 1 < L.H && inside(x, y + 1)) b |= MASK_GY;
         host[(size_t)y * L.P + x] = b;
       }
-    FS_CUDA(cudaMemcpy((void*)L.v.mask, host.data(), host.size(), cudaMemcpyHostToDevice));
+    // on the handle's stream, behind the clearing of the arena (the stream
+    // may be a non-blocking one, which the legacy stream does not wait for);
+    // the host buffer is filled again for the next level
+    FS_CUDA(cudaMemcpyAsync((void*)L.v.mask, host.data(), host.size(), cudaMemcpyHostToDevice,
+                            h->stream));
+    FS_CUDA(cudaStreamSynchronize(h->stream));
   }
   return FS_OK;
 }
@@ -488,8 +493,9 @@ fs_status ensure_schedule(fs_handle* h, int iters) {
     t *= th;
     s /= th;
   }
+  FS_CUDA(cudaMemcpyAsync(h->sched, tab.data(), tab.size() * sizeof(float4),
+                          cudaMemcpyHostToDevice, h->stream));
   FS_CUDA(cudaStreamSynchronize(h->stream));
-  FS_CUDA(cudaMemcpy(h->sched, tab.data(), tab.size() * sizeof(float4), cudaMemcpyHostToDevice));
   h->sched_iters = iters;
   return FS_OK;
 }
