@@ -91,11 +91,12 @@ typedef struct {
  * over-relaxation of Eq. 11 (1 = Chambolle-Pock Algorithm 1).  precond = 1
  * uses diagonal preconditioning (Pock-Chambolle 2011, alpha = 1), 0 uses
  * tau = sigma = 1/sqrt(8).  block_iters: primal-dual iterations fused per
- * launch by temporal blocking (1..8; 0 = library default).  use_graph = 1
+ * launch by temporal blocking (1..8; 0 = chosen by level size).  use_graph = 1
  * captures a solve into a CUDA graph on first use and replays it.
- * pd_schedule: 0 = automatic (levels up to 128 x 128 run all iterations of
- * a warp in one launch of a thread-block cluster holding the whole level,
- * when the GPU can host that cluster; larger levels use temporal blocking),
+ * pd_schedule: 0 = automatic (temporal blocking with footprint and depth
+ * chosen by level size and iterations; in 16-bit storage levels up to
+ * 128 x 128 run all iterations of a warp in one launch of a thread-block
+ * cluster holding the whole level, when the GPU can host that cluster),
  * 1 = temporal blocking on every level, FS_SCHED_PERSISTENT (2) = the
  * persistent schedule: after the pre-rotation and the pyramid, every level
  * and warp of a cold solve -- and, in fs_batch_solve, of every pair of the

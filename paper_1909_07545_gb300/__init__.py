@@ -355,8 +355,10 @@ class Solver:
         threads, 32x32 of 256, 64x32 of 256, 64x64 of 1024, 32x32 of 1024,
         32x32 of 512), so 1..48; 49..55 = depth 9..15 on 32x32 of 1024
         threads; 56..63 = depth 1..8 on the TMA-staged 64x64 footprints;
-        64..71 = depth 1..8 on 64x48 of 768 threads.  TGV handles: 0 = a
-        launch per step, 8 v + d = depth d on the five TGV footprints."""
+        64..71 = depth 1..8 on 64x48 of 768 threads.  (Where the automatic
+        schedule is faster than all of them the handle keeps that, and the
+        best of these is returned.)  TGV handles: 0 = a launch per step,
+        8 v + d = depth d on the five TGV footprints."""
         out = (ctypes.c_int * 8)()
         _check(self.lib.fs_autotune(self.h, int(iters), out))
         return [out[l] for l in range(self.levels)]

@@ -66,6 +66,7 @@ struct HostLevel {
   int cluster = -1;                         // whole-level cluster variant, -1 if none
   int tuned = -1;                           // autotuned choice: 0 cluster, 1..8 depth, -1 none
   int tuned_variant = -1;                   // autotuned tile variant, -1: by size
+  bool auto_best = false;                   // the tuner found pd_auto's schedule faster still
   LevelView v{};
   // tensor maps of the TMA-staged primal-dual footprints, reading buffer
   // set 0 (primary) and set 1 (alternate); tma_ok = false if the driver
@@ -246,6 +247,7 @@ struct fs_handle {
   fs_pose pose;
   fs_params prm;
   int W = 0, H = 0, L = 0;
+  int sms = 0;                            // SMs of the device
   cudaStream_t stream = nullptr;
   cudaStream_t cap_stream = nullptr;
   HostLevel lv[kMaxLevels];
@@ -388,17 +390,6 @@ fs_status build_fields(fs_handle* h) {
   return FS_OK;
 }
 
-// Iterations fused per k_pd launch (temporal-blocking depth).  0 picks by
-// level size: 6 for levels wider than 512 px, where the halo recomputation
-// starts to cost more than the saved launches, 8 below (launch-latency
-// bound); measured on GB300 with the 1024 x 1024 workload.
-int pd_block(const fs_handle* h, int l) {
-  int b = h->prm.block_iters;
-  if (b <= 0 && h->lv[l].tuned >= 1) return h->lv[l].tuned;
-  if (b <= 0) return (h->lv[l].W > 512 || h->lv[l].H > 512) ? 6 : 8;
-  return b > 8 ? 8 : b;
-}
-
 // A schedule choice of fs_autotune / fs_set_schedule: 0 = cluster (Huber-TV)
 // or a launch per step (TGV); 8 v + 1 .. 8 v + 8 = blocking depth 1..8 on
 // footprint variant v (PDVariant: 64 x 64 of 512 threads, 32 x 32 of 256,
@@ -436,30 +427,45 @@ void decode_choice(int c, bool tgv, int& depth, int& variant) {
   variant = (c - 1) / 8;
 }
 
-// Whether level l runs the whole-level cluster schedule.
+// Whether level l runs the whole-level cluster schedule: when it was chosen
+// (fs_set_schedule, the tuner), and by default in 16-bit storage, where
+// temporal blocking would round the dual at every launch.  In FP32 blocking
+// gives the same bits in less than half the time (128 x 128, 100
+// iterations: 47 us against 119).
 bool use_cluster(const fs_handle* h, int l) {
   const HostLevel& L = h->lv[l];
   if (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0) return false;
   if (h->prm.block_iters <= 0 && L.tuned >= 1) return false;   // tuner chose blocking
-  return true;
+  return L.tuned == 0 && !L.auto_best ? true : h->prm.storage != ST_F32;
+}
+
+// The temporal-blocking launches of `iters` iterations on level l: the tuned
+// choice, else pd_auto.  block_iters, when set, fixes the number of
+// launches, and so does 16-bit storage (depth 6 on levels wider than 512 px,
+// 8 below), whose results depend on it.  A halo is never deeper than the
+// longest launch's iterations.
+PdSchedule pd_plan(const fs_handle* h, int l, int iters) {
+  const HostLevel& L = h->lv[l];
+  const int b = std::min(h->prm.block_iters, 8);
+  if (b <= 0 && L.tuned >= 1 && !L.auto_best) {
+    const int nl = pd_launch_count(iters, L.tuned);
+    return PdSchedule{L.tuned_variant, nl, (iters + nl - 1) / nl};
+  }
+  int nl = 0;
+  if (h->prm.storage != ST_F32)
+    nl = pd_launch_count(iters, b > 0 ? b : (L.W > 512 || L.H > 512) ? 6 : 8);
+  else if (b > 0 && (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0))
+    nl = pd_launch_count(iters, b);
+  return pd_auto(L.W, L.H, iters, nl, h->sms);
 }
 
 // Whether a solve of h runs the TMA-staged footprints on some level.
 bool uses_tma(const fs_handle* h) {
   if (h->prm.regularizer == FS_REG_TGV || h->prm.block_iters > 0) return false;
   for (int l = 0; l < h->L; ++l)
-    if (h->lv[l].tuned >= 1 && h->lv[l].tuned_variant == PD_TILE_64_TMA) return true;
+    if (h->lv[l].tuned >= 1 && !h->lv[l].auto_best && h->lv[l].tuned_variant == PD_TILE_64_TMA)
+      return true;
   return false;
-}
-
-// Number of k_pd launches for `iters` iterations with at most B per launch:
-// ceil(iters / B), raised to an even count (when iters >= 2) so that the
-// ping-pong state ends in the primary buffers (a launch may then run 0
-// iterations, i.e. only copy its interior across).
-int pd_launches(int iters, int B) {
-  int n = (iters + B - 1) / B;
-  if (n % 2 == 1 && iters >= 2) ++n;
-  return n;
 }
 
 // The accelerated schedule's table for at least `iters` iterations per
@@ -523,10 +529,8 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st) {
       return fail(FS_ECUDA, "launch of k_pd_cluster failed: %s", cudaGetErrorString(e));
     return FS_OK;
   }
-  int B = pd_block(h, l);
-  int variant = L.tuned_variant >= 0 && h->prm.block_iters <= 0
-                    ? L.tuned_variant
-                    : ((L.W >= 128 && L.H >= 128) ? PD_TILE_64 : PD_TILE_32);
+  const PdSchedule ps = pd_plan(h, l, iters);
+  const int variant = ps.variant, B = ps.depth, nl = ps.launches;
   PDState A{L.v.u, L.v.ubar, L.v.p1, L.v.p2};
   PDState Bs{L.v.u_alt, L.v.ubar_alt, L.v.p1_alt, L.v.p2_alt};
   const bool tma = variant == PD_TILE_64_TMA;
@@ -535,7 +539,6 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st) {
     FS_LAUNCH("k_pd_consts", launch_pd_consts(L.v, h->prm.lambda, h->prm.huber_eps, st));
     L.consts_stale = false;
   }
-  int nl = pd_launches(iters, B);
   for (int k = 0, done = 0; k < nl; ++k) {
     int n = (iters - done) / (nl - k);          // spread the iterations evenly
     if ((iters - done) % (nl - k)) ++n;
@@ -1078,6 +1081,12 @@ fs_status fs_create(const fs_calib cam[2], const fs_pose* pose, int W, int H, in
   h->H = H;
   h->L = levels;
   h->stream = (cudaStream_t)cuda_stream;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    h->sms = 152;                       // the allocation below reports what is wrong
+  }
 
   // level sizes and scaled calibrations (f 2^-l, (c + 0.5) 2^-l - 0.5)
   size_t bytes = 0;
@@ -1660,7 +1669,11 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
   if (choice) *choice = -1;
   const int n = (int)b->h.size();
   // every handle's own coarse choices (to restore when they win)
-  std::vector<std::vector<std::pair<int, int>>> own(n);
+  struct Own {
+    int tuned, variant;
+    bool auto_best;
+  };
+  std::vector<std::vector<Own>> own(n);
   bool any = false;
   for (int i = 0; i < n; ++i) {
     fs_handle* h = b->h[i];
@@ -1669,7 +1682,7 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
     fs_status s;
     if ((s = ensure_schedule(h, iters)) != FS_OK) return s;
     for (int l = 2; l < h->L; ++l) {
-      own[i].push_back({h->lv[l].tuned, h->lv[l].tuned_variant});
+      own[i].push_back({h->lv[l].tuned, h->lv[l].tuned_variant, h->lv[l].auto_best});
       any = true;
     }
   }
@@ -1685,9 +1698,11 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
       for (int l = 2; l < h->L; ++l) {
         HostLevel& L = h->lv[l];
         if (c < 0) {
-          L.tuned = own[i][l - 2].first;
-          L.tuned_variant = own[i][l - 2].second;
+          L.tuned = own[i][l - 2].tuned;
+          L.tuned_variant = own[i][l - 2].variant;
+          L.auto_best = own[i][l - 2].auto_best;
         } else {
+          L.auto_best = false;
           decode_choice(c, false, L.tuned, L.tuned_variant);
         }
       }
@@ -1904,7 +1919,6 @@ extern "C" fs_status fs_timing_read(fs_handle* h, double* ms, long long* launche
   if (h->ev_pending) {
     FS_CUDA(cudaStreamSynchronize(h->stream));
     for (int l = 0; l < h->ev_levels; ++l) {
-      int B = pd_block(h, l);
       for (int w = 0; w < h->ev_warps; ++w) {
         float t = 0.f;
         FS_CUDA(cudaEventElapsedTime(&t, h->ev[2 * (l * h->ev_warps + w)],
@@ -1913,7 +1927,7 @@ extern "C" fs_status fs_timing_read(fs_handle* h, double* ms, long long* launche
       }
       h->t_launch[l] += use_cluster(h, l)
                             ? (long long)h->ev_warps
-                            : (long long)h->ev_warps * pd_launches(h->ev_iters, B);
+                            : (long long)h->ev_warps * pd_plan(h, l, h->ev_iters).launches;
       h->t_pxit[l] += (double)h->lv[l].W * h->lv[l].H * h->ev_warps * h->ev_iters;
     }
     h->ev_pending = false;
@@ -1944,15 +1958,12 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
     HostLevel& L = h->lv[l];
     L.tuned = -1;
     L.tuned_variant = -1;
+    L.auto_best = false;
     float best = 3.4e38f;
     int best_c = -1;
     std::vector<float> timed(kMaxChoice + 1, -1.f);
-    // best of 3 timed runs after a warm-up, each candidate once
-    auto try_cand = [&](int cand) {
-      if (st != FS_OK || timed[cand] >= 0.f) return;
-      h->prm.pd_schedule = cand == 0 ? 0 : 1;
-      h->prm.block_iters = saved_block;
-      decode_choice(cand, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
+    // best of 3 timed runs of the level's schedule as it stands, after a warm-up
+    auto time_level = [&]() {
       float t = 3.4e38f;
       for (int rep = 0; rep < 4 && st == FS_OK; ++rep) {
         cudaError_t e = cudaEventRecord(e0, h->stream);
@@ -1964,6 +1975,15 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
         if (e != cudaSuccess) { st = fail(FS_ECUDA, "fs_autotune: %s", cudaGetErrorString(e)); break; }
         if (rep > 0 && ms < t) t = ms;
       }
+      return t;
+    };
+    // each candidate once
+    auto try_cand = [&](int cand) {
+      if (st != FS_OK || timed[cand] >= 0.f) return;
+      h->prm.pd_schedule = cand == 0 ? 0 : 1;
+      h->prm.block_iters = saved_block;
+      decode_choice(cand, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
+      const float t = time_level();
       timed[cand] = t;
       if (st == FS_OK && t < best) { best = t; best_c = cand; }
     };
@@ -1980,7 +2000,17 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
       for (int cand = 1; cand <= kMaxChoice; ++cand)
         if (L.tma_ok || !is_tma_choice(cand, false)) try_cand(cand);
     }
+    // the automatic schedule, whose footprints and depths go beyond the
+    // encoding: where it is faster still, the handle keeps it and `choice`
+    // reports the best encoded one
+    bool auto_best = false;
+    if (h->prm.regularizer != FS_REG_TGV && saved_block <= 0 && st == FS_OK) {
+      h->prm.pd_schedule = saved_sched == 0 ? 0 : 1;
+      L.tuned = L.tuned_variant = -1;
+      auto_best = time_level() < best;
+    }
     decode_choice(best_c, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
+    L.auto_best = auto_best;
     if (choice) choice[l] = best_c;
   }
   h->prm.block_iters = saved_block;
@@ -2034,6 +2064,7 @@ extern "C" fs_status fs_set_schedule(fs_handle* h, const int* choice) {
     int c = choice[l];
     HostLevel& L = h->lv[l];
     decode_choice(c, tgv, L.tuned, L.tuned_variant);
+    L.auto_best = false;
   }
   return FS_OK;
 }

@@ -26,6 +26,20 @@ constexpr int PD_TILE_64_TMA = PD_TILE_COUNT;
 // at depth 6 has 150 of them, one per SM, where 64 x 64 footprints leave
 // 31 SMs idle.
 constexpr int PD_TILE_64x48_T768 = PD_TILE_COUNT + 1;
+// Footprints only the automatic schedule (pd_auto) uses, also launch_pd
+// variants.  Between 32 x 32 and 64 x 48 they fill the steps at which a
+// level fits one footprint per SM with the deepest halo: 100 iterations of a
+// 256 x 256 level take 57 us on 32 x 48 against 65 us on the best of the
+// others, of 320 x 320 67 against 78, of 64 x 64 39 (32 x 24) against 44.
+// 64 x 32 of 512 threads runs two CTAs per SM, whose loads, barriers and
+// iterations overlap: 1024 x 1024 takes 392 us against 415 (64 x 64 of 1024
+// threads), 2048 x 2048 1630 against 1900.
+constexpr int PD_TILE_32x16_T256 = PD_TILE_COUNT + 2;
+constexpr int PD_TILE_32x24_T384 = PD_TILE_COUNT + 3;
+constexpr int PD_TILE_32x48_T768 = PD_TILE_COUNT + 4;
+constexpr int PD_TILE_64x24_T768 = PD_TILE_COUNT + 5;
+constexpr int PD_TILE_64x32_T1024 = PD_TILE_COUNT + 6;
+constexpr int PD_TILE_64x32_T512 = PD_TILE_COUNT + 7;
 enum PDClusterVariant { PD_CLUSTER_16 = 0, PD_CLUSTER_32 = 1 };
 
 __global__ void k_trajectory(DevCamDF cam, df tx, df ty, df tz, LevelView L);
@@ -103,6 +117,19 @@ cudaError_t launch_pd_consts(const LevelView& L, float lam, float eps, cudaStrea
 // before reading the state.
 cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const PDState& out,
                       const PDParams& pp, int B, int n, cudaStream_t st, bool chained = false);
+
+// The automatic schedule of `iters` iterations on a W x H level: a footprint
+// (variant), the number of launches and the halo depth (the iterations of
+// the longest launch).  launches > 0 fixes the number of launches (16-bit
+// storage rounds the dual at each launch's end, so there it is part of the
+// result); 0 leaves it free.
+struct PdSchedule {
+  int variant, launches, depth;
+};
+PdSchedule pd_auto(int W, int H, int iters, int launches, int sms);
+// Launches of `iters` iterations at most `depth` each, made even when
+// iters >= 2 so that the ping-pong state ends where it began.
+int pd_launch_count(int iters, int depth);
 
 // The tensor maps k_pd_tma copies a footprint through: T^1/2, tau, the
 // per-warp constants (launch_pd_consts) and the mask of a level, and the

@@ -163,21 +163,24 @@ extern "C" fs_status fs_pd_iterate_noalloc(const float* d_I0, const unsigned cha
     return fs_internal_set_error(FS_ECUDA, msg);
   }
 
-  // same launch schedule as the handle path: at most B iterations per
-  // launch, an even number of launches so the state ends in the caller's
-  // buffers
-  int B = p.block_iters <= 0 ? 4 : p.block_iters;
-  int nl = (iters + B - 1) / B;
-  if (nl % 2 == 1 && iters >= 2) ++nl;
-  int variant = (W >= 128 && H >= 128) ? PD_TILE_64 : PD_TILE_32;
+  // same launch schedule as the handle path: an even number of launches, so
+  // the state ends in the caller's buffers, each but the first chained to
+  // the one before (the constants were written before the first)
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const PdSchedule ps =
+      pd_auto(W, H, iters, p.block_iters > 0 ? pd_launch_count(iters, p.block_iters) : 0, sms);
+  const int nl = ps.launches;
   PDParams pp{p.lambda, p.huber_eps, p.theta};
   PDState A{L.u, L.ubar, L.p1, L.p2};
   PDState Bs{L.u_alt, L.ubar_alt, L.p1_alt, L.p2_alt};
-  for (int k = 0, done = 0; k < nl; ++k) {
+  for (int k = 0, done = 0; k < nl && e == cudaSuccess; ++k) {
     int m = (iters - done) / (nl - k);
     if ((iters - done) % (nl - k)) ++m;
-    e = launch_pd(variant, L, (k % 2 == 0) ? A : Bs, (k % 2 == 0) ? Bs : A, pp, B, m, st);
-    if (e != cudaSuccess) break;
+    e = launch_pd(ps.variant, L, (k % 2 == 0) ? A : Bs, (k % 2 == 0) ? Bs : A, pp, ps.depth, m,
+                  st, k > 0);
     done += m;
   }
   if (e == cudaSuccess && nl % 2 == 1) {

@@ -4,11 +4,11 @@
 //
 // 1. k_pd -- temporal blocking, for levels too large to stay on chip: one
 //    CTA per footprint, the body in pd_tile.cuh (an interior tile plus a halo
-//    of B pixels, n <= B iterations per launch).  Six footprints (PDVariant)
-//    trade registers per thread (R rows) against resident warps and halo
-//    recomputation; the autotuner picks one per level.  ACC instantiations
-//    read the accelerated step schedule, one table entry per iteration of
-//    the warp.
+//    of B pixels, n <= B iterations per launch).  The footprints trade
+//    registers per thread (R rows) against resident warps and halo
+//    recomputation; pd_auto or the autotuner picks one per level.  ACC
+//    instantiations read the accelerated step schedule, one table entry per
+//    iteration of the warp.
 //
 // 2. k_pd_cluster -- the whole level resident in one thread-block cluster
 //    (at most 16 CTAs, one tile each, no halo), for the coarse levels.  Each
@@ -19,6 +19,9 @@
 //
 // grad: forward differences masked by MASK_GX / MASK_GY; div: its exact
 // negative adjoint; u is only updated inside the FOV mask.
+#include <algorithm>
+#include <cmath>
+
 #include <cooperative_groups.h>
 
 #include "fs_kernels.h"
@@ -57,8 +60,9 @@ cudaError_t launch_pd_consts(const LevelView& L, float lam, float eps, cudaStrea
   return cudaGetLastError();
 }
 
-template <int FW, int NY, int R, int S, bool ACC>
-__global__ void __launch_bounds__(FW * NY, FW * NY >= 512 ? 1 : 2)
+// MB: CTAs per SM the registers have to allow.
+template <int FW, int NY, int R, int S, bool ACC, int MB>
+__global__ void __launch_bounds__(FW * NY, MB)
 k_pd(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, int chained) {
   constexpr int FH = NY * R;
   __shared__ float s_ub[FH][FW];
@@ -188,7 +192,7 @@ k_pd_cluster(LevelView L, PDParams pp, int n_iters) {
   }
 }
 
-template <int FW, int NY, int R, int S, bool ACC = false>
+template <int FW, int NY, int R, int S, bool ACC, int MB = (FW * NY >= 512 ? 1 : 2)>
 static cudaError_t launch_pd_t(const LevelView& L, const PDState& in, const PDState& out,
                                const PDParams& pp, int B, int n, bool chained,
                                cudaStream_t st) {
@@ -203,54 +207,109 @@ static cudaError_t launch_pd_t(const LevelView& L, const PDState& in, const PDSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_pd<FW, NY, R, S, ACC>, L, in, out, pp, B, n, chained ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, k_pd<FW, NY, R, S, ACC, MB>, L, in, out, pp, B, n, chained ? 1 : 0);
 }
 
-template <int S>
+template <int S, bool ACC>
 static cudaError_t launch_pd_s(int variant, const LevelView& L, const PDState& in,
                                const PDState& out, const PDParams& pp, int B, int n,
                                cudaStream_t st, bool chained) {
+#define FS_PD(...) return launch_pd_t<__VA_ARGS__>(L, in, out, pp, B, n, chained, st)
   switch (variant) {
-    case PD_TILE_64: return launch_pd_t<64, 8, 8, S>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_32: return launch_pd_t<32, 8, 4, S>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_64x32: return launch_pd_t<64, 4, 8, S>(L, in, out, pp, B, n, chained, st);
+    case PD_TILE_64: FS_PD(64, 8, 8, S, ACC);
+    case PD_TILE_32: FS_PD(32, 8, 4, S, ACC);
+    case PD_TILE_64x32: FS_PD(64, 4, 8, S, ACC);
     // the 64 x 64 footprint with 1024 threads of 4 rows (64 registers):
     // twice the resident warps of 512 threads of 8 rows
-    case PD_TILE_64_T1024: return launch_pd_t<64, 16, 4, S>(L, in, out, pp, B, n, chained, st);
+    case PD_TILE_64_T1024: FS_PD(64, 16, 4, S, ACC);
     // small levels: the 32 x 32 footprint spread over more threads, which
     // shortens each thread's dependent chain per iteration (the small levels
     // are latency-bound, not issue-bound)
-    case PD_TILE_32_T1024: return launch_pd_t<32, 32, 1, S>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_32_T512: return launch_pd_t<32, 16, 2, S>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_64x48_T768: return launch_pd_t<64, 12, 4, S>(L, in, out, pp, B, n, chained, st);
+    case PD_TILE_32_T1024: FS_PD(32, 32, 1, S, ACC);
+    case PD_TILE_32_T512: FS_PD(32, 16, 2, S, ACC);
+    case PD_TILE_64x48_T768: FS_PD(64, 12, 4, S, ACC);
+    case PD_TILE_32x16_T256: FS_PD(32, 8, 2, S, ACC);
+    case PD_TILE_32x24_T384: FS_PD(32, 12, 2, S, ACC, 1);
+    case PD_TILE_32x48_T768: FS_PD(32, 24, 2, S, ACC);
+    case PD_TILE_64x24_T768: FS_PD(64, 12, 2, S, ACC);
+    case PD_TILE_64x32_T1024: FS_PD(64, 16, 2, S, ACC);
+    case PD_TILE_64x32_T512: FS_PD(64, 8, 4, S, ACC, 2);
     default: return cudaErrorInvalidValue;
   }
+#undef FS_PD
 }
 
-// The accelerated schedule (FP32 storage only) on each footprint.
-static cudaError_t launch_pd_acc(int variant, const LevelView& L, const PDState& in,
-                                 const PDState& out, const PDParams& pp, int B, int n,
-                                 cudaStream_t st, bool chained) {
-  if (L.st != ST_F32) return cudaErrorInvalidValue;
-  switch (variant) {
-    case PD_TILE_64: return launch_pd_t<64, 8, 8, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_32: return launch_pd_t<32, 8, 4, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_64x32: return launch_pd_t<64, 4, 8, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_64_T1024: return launch_pd_t<64, 16, 4, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_32_T1024: return launch_pd_t<32, 32, 1, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_32_T512: return launch_pd_t<32, 16, 2, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    case PD_TILE_64x48_T768: return launch_pd_t<64, 12, 4, ST_F32, true>(L, in, out, pp, B, n, chained, st);
-    default: return cudaErrorInvalidValue;
+int pd_launch_count(int iters, int depth) {
+  int n = (iters + depth - 1) / depth;
+  if (n % 2 == 1 && iters >= 2) ++n;
+  return n;
+}
+
+// The least of the modelled times over footprints and launch counts.  A
+// launch of n iterations takes t0 + n b microseconds per wave of CTAs (per_sm
+// of them on every SM): t0 the launch, the loads and the stores, b one
+// iteration, both fitted to the sizes of the table below on GB300 (graph
+// replays, warm).  What the rule picks against the fixed choice it replaces
+// (64 x 64 footprints of 512 threads at depth 8, at depth 6 above 512 pixels,
+// 32 x 32 of 256 threads below 128), us per 10 / 100 iterations:
+//   64 x 64     5.8 / 39.4   against   7.4 / 49.2
+//   128 x 128   6.0 / 46.9            16.5 / 125.7
+//   256 x 256   8.0 / 56.9            16.9 / 128.3
+//   400 x 400  11.0 / 85.5            17.1 / 128.4
+//   640 x 640  18.7 / 156.4           31.4 / 276.2
+//   1024 x 1024  41.9 / 392           47.5 / 434
+//   2048 x 2048 (50 iterations)  816          1034
+PdSchedule pd_auto(int W, int H, int iters, int launches, int sms) {
+  struct Fit {
+    int variant, fw, fh, per_sm;
+    float t0, b;
+  };
+  static const Fit kFit[] = {
+      {PD_TILE_32x16_T256, 32, 16, 1, 1.95f, 0.18f}, {PD_TILE_32x24_T384, 32, 24, 1, 1.85f, 0.185f},
+      {PD_TILE_32_T512, 32, 32, 1, 1.7f, 0.245f},    {PD_TILE_32_T1024, 32, 32, 1, 1.86f, 0.282f},
+      {PD_TILE_32x48_T768, 32, 48, 1, 1.95f, 0.31f}, {PD_TILE_64x24_T768, 64, 24, 1, 1.9f, 0.315f},
+      {PD_TILE_64x32_T1024, 64, 32, 1, 2.4f, 0.37f}, {PD_TILE_64x48_T768, 64, 48, 1, 3.0f, 0.55f},
+      {PD_TILE_64_T1024, 64, 64, 1, 4.1f, 0.735f},   {PD_TILE_64x32_T512, 64, 32, 2, 3.2f, 0.67f},
+  };
+  constexpr int kMaxDepth = 15;
+  PdSchedule best{PD_TILE_32_T512, launches > 0 ? launches : pd_launch_count(iters, 8), 0};
+  double best_us = 1e300;
+  auto consider = [&](int nl) {
+    const int depth = std::max(1, (iters + nl - 1) / nl);
+    if (depth > kMaxDepth) return;
+    for (const Fit& f : kFit) {
+      const int iw = f.fw - 2 * depth, ih = f.fh - 2 * depth;
+      if (iw < 2 || ih < 2) continue;
+      const double tiles = (double)((W + iw - 1) / iw) * ((H + ih - 1) / ih);
+      const double waves = std::ceil(tiles / ((double)f.per_sm * sms));
+      const double us = nl * waves * (f.t0 + f.b * iters / nl);
+      if (us < best_us) {
+        best_us = us;
+        best = PdSchedule{f.variant, nl, depth};
+      }
+    }
+  };
+  if (launches > 0) {
+    consider(launches);
+  } else if (iters < 2) {
+    consider(1);
+  } else {
+    for (int depth = kMaxDepth; depth >= 3; --depth) consider(pd_launch_count(iters, depth));
   }
+  if (best.depth == 0) best.depth = std::max(1, (iters + best.launches - 1) / best.launches);
+  return best;
 }
 
 cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const PDState& out,
                       const PDParams& pp, int B, int n, cudaStream_t st, bool chained) {
-  if (pp.sched) return launch_pd_acc(variant, L, in, out, pp, B, n, st, chained);
+  if (pp.sched) {                       // the accelerated schedule: FP32 storage only
+    if (L.st != ST_F32) return cudaErrorInvalidValue;
+    return launch_pd_s<ST_F32, true>(variant, L, in, out, pp, B, n, st, chained);
+  }
   switch (L.st) {
-    case ST_F16: return launch_pd_s<ST_F16>(variant, L, in, out, pp, B, n, st, chained);
-    case ST_BF16: return launch_pd_s<ST_BF16>(variant, L, in, out, pp, B, n, st, chained);
-    default: return launch_pd_s<ST_F32>(variant, L, in, out, pp, B, n, st, chained);
+    case ST_F16: return launch_pd_s<ST_F16, false>(variant, L, in, out, pp, B, n, st, chained);
+    case ST_BF16: return launch_pd_s<ST_BF16, false>(variant, L, in, out, pp, B, n, st, chained);
+    default: return launch_pd_s<ST_F32, false>(variant, L, in, out, pp, B, n, st, chained);
   }
 }
 
