@@ -20,6 +20,7 @@
 #include "pd_tgv_math.cuh"
 #include "fs_stages.h"
 #include "fs_kernels.h"
+#include "pd_tile.cuh"
 
 using namespace fs;
 
@@ -468,6 +469,18 @@ bool uses_tma(const fs_handle* h) {
   return false;
 }
 
+// Whether a warp's launches on level l -- the warp start, the iterations, the
+// clip -- form one chain of programmatic dependent launches: when they are
+// few, so that the gaps between them count.  (10 iterations on each of 5
+// levels of 800 x 800, 2 launches a warp: 1.87 -> 1.78 ms a frame; 20 on 3
+// levels of 128 x 128: 211 -> 170 us.  With 8 launches a warp the chain's
+// reading of the constants through L2 costs more than the gaps, 505 -> 526
+// us on 256 x 256; with 4 it still loses 2 %.)
+bool short_chain(const fs_handle* h, int l, int iters) {
+  return h->prm.regularizer == FS_REG_HUBER_TV && !use_cluster(h, l) &&
+         pd_plan(h, l, iters).launches <= 2;
+}
+
 // The accelerated schedule's table for at least `iters` iterations per
 // warp, built in FP64 on the host and stored as FP32 (synchronous; called
 // outside any graph capture, before the launches that read it).  The table
@@ -506,7 +519,9 @@ fs_status ensure_schedule(fs_handle* h, int iters) {
   return FS_OK;
 }
 
-fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st) {
+// chain: the launch before on the stream is this library's warp start of the
+// level (the first launch may then be a programmatic dependent one).
+fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = false) {
   HostLevel& L = h->lv[l];
   PDParams pp{h->prm.lambda, h->prm.huber_eps, h->prm.theta};
   if (h->prm.accel_gamma > 0) {
@@ -535,6 +550,7 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st) {
   PDState Bs{L.v.u_alt, L.v.ubar_alt, L.v.p1_alt, L.v.p2_alt};
   const bool tma = variant == PD_TILE_64_TMA;
   if (tma && !L.tma_ok) return fail(FS_EINVAL, "level %d: no tensor maps for the TMA footprints", l);
+  pp.fresh = chain && !L.consts_stale && short_chain(h, l, iters);
   if (L.consts_stale) {
     FS_LAUNCH("k_pd_consts", launch_pd_consts(L.v, h->prm.lambda, h->prm.huber_eps, st));
     L.consts_stale = false;
@@ -545,9 +561,10 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st) {
     const PDState& in = (k % 2 == 0) ? A : Bs;
     const PDState& out = (k % 2 == 0) ? Bs : A;
     pp.k0 = done;
-    cudaError_t e = tma ? launch_pd_tma(L.v, out, pp, B, n, k > 0, L.tma[k % 2], h->pd_status,
+    const int link = k > 0 ? PD_CHAINED : pp.fresh ? PD_CHAIN_START : 0;
+    cudaError_t e = tma ? launch_pd_tma(L.v, out, pp, B, n, link, L.tma[k % 2], h->pd_status,
                                         h->wait_ns, (h->persist_stall && k == 0) ? 1 : 0, st)
-                        : launch_pd(variant, L.v, in, out, pp, B, n, st, k > 0);
+                        : launch_pd(variant, L.v, in, out, pp, B, n, st, link);
     if (e != cudaSuccess)
       return fail(FS_ECUDA, "launch of %s failed: %s", tma ? "k_pd_tma" : "k_pd",
                   cudaGetErrorString(e));
@@ -564,7 +581,10 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st) {
   return FS_OK;
 }
 
-fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st) {
+// chain: FS_STAGE_CLIP and FS_STAGE_CLIP_WARP directly behind run_pd's
+// launches on the stream.
+fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
+                    bool chain = false) {
   HostLevel& L = h->lv[l];
   const int consts = h->prm.regularizer == FS_REG_TGV ? 0 : 1;
   // every stage but the iterations and the warp starts can change sigma,
@@ -597,13 +617,12 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st) 
       return s != FS_OK ? s : run_pd(h, l, count, st);
     }
     case FS_STAGE_CLIP:
-      k_clip<<<grid2(L.W, L.H), kBlock2, 0, st>>>(L.v, h->prm.du_max);
-      FS_LAUNCHED("k_clip");
+      FS_LAUNCH("k_clip", launch_clip(L.v, h->prm.du_max, chain, st));
       return FS_OK;
     case FS_STAGE_CLIP_WARP:
       FS_LAUNCH("k_clip_warp", launch_clip_warp(L.v, h->prm.du_max,
                                                 h->prm.deriv == FS_DERIV_CENTRAL, h->prm.lambda,
-                                                h->prm.huber_eps, consts, st));
+                                                h->prm.huber_eps, consts, chain, st));
       L.consts_stale = !consts;
       if (h->prm.regularizer == FS_REG_TGV)
         FS_LAUNCH("k_tgv_warp_start", launch_tgv_warp_start(L.v, st));
@@ -621,8 +640,9 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st) 
 
 // The end of a warp (clip + update, Eq. 8-9) and, when another warp
 // follows, its start (warp + linearise) in one fused launch.
-fs_status clip_then_warp(fs_handle* h, int l, bool next, cudaStream_t st) {
-  return run_stage(h, l, next ? FS_STAGE_CLIP_WARP : FS_STAGE_CLIP, 0, st);
+fs_status clip_then_warp(fs_handle* h, int l, int iters, bool next, cudaStream_t st) {
+  return run_stage(h, l, next ? FS_STAGE_CLIP_WARP : FS_STAGE_CLIP, 0, st,
+                   short_chain(h, l, iters));
 }
 
 fs_status enqueue_depth(fs_handle* h, float* disp, float* depth, cudaStream_t st) {
@@ -673,9 +693,9 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     if ((s = run_stage(h, 0, FS_STAGE_WARP, 0, st)) != FS_OK) return s;
     for (int w = 0; w < warps; ++w) {
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w], st));
-      if ((s = run_pd(h, 0, iters, st)) != FS_OK) return s;
+      if ((s = run_pd(h, 0, iters, st, true)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w + 1], st));
-      if ((s = clip_then_warp(h, 0, w + 1 < warps, st)) != FS_OK) return s;
+      if ((s = clip_then_warp(h, 0, iters, w + 1 < warps, st)) != FS_OK) return s;
     }
     if (h->timing) {
       h->ev_warps = warps;
@@ -705,9 +725,9 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     if ((s = run_stage(h, l, FS_STAGE_WARP, 0, st)) != FS_OK) return s;
     for (int w = 0; w < warps; ++w) {
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w)], st));
-      if ((s = run_pd(h, l, iters, st)) != FS_OK) return s;
+      if ((s = run_pd(h, l, iters, st, true)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w) + 1], st));
-      if ((s = clip_then_warp(h, l, w + 1 < warps, st)) != FS_OK) return s;
+      if ((s = clip_then_warp(h, l, iters, w + 1 < warps, st)) != FS_OK) return s;
     }
   }
   if (h->timing) {

@@ -352,6 +352,7 @@ struct PDParams {
   // done before this launch.
   const float4* sched = nullptr;
   int k0 = 0;
+  int fresh = 0;        // the chain of launches starts with PD_CHAIN_START
 };
 
 }  // namespace fs

@@ -47,7 +47,6 @@ __global__ void k_calib_field(DevCamDF c0, DevCamDF c1, RotDF R, const uint8_t* 
                               float4* __restrict__ field, int W, int H, int P);
 __global__ void k_copy_in(const float* __restrict__ src, float* __restrict__ dst, int W, int H,
                           int P);
-__global__ void k_clip(LevelView L, float du_max);
 __global__ void k_depth(LevelView L, DevCam cam, float Cx, float Cy, float Cz,
                         float* __restrict__ disp, float* __restrict__ depth);
 __global__ void k_pack(const float* __restrict__ src, int stride, float* __restrict__ dst, int W,
@@ -93,9 +92,13 @@ cudaError_t launch_tensor(const LevelView& L, float beta, float eta, int precond
 // kernel writes.
 cudaError_t launch_warp(const LevelView& L, int central, float lam, float eps, int consts,
                         cudaStream_t st);
-// k_clip of one warp fused with k_warp of the next (same results).
+// k_clip of one warp fused with k_warp of the next (same results).  chained:
+// a programmatic dependent launch behind the warp's iterations, which waits
+// for them before it reads anything they or the last warp start wrote; so for
+// k_clip.
 cudaError_t launch_clip_warp(const LevelView& L, float du_max, int central, float lam, float eps,
-                             int consts, cudaStream_t st);
+                             int consts, bool chained, cudaStream_t st);
+cudaError_t launch_clip(const LevelView& L, float du_max, bool chained, cudaStream_t st);
 cudaError_t launch_tensor_abc(const LevelView& L, float* dst, cudaStream_t st);
 cudaError_t launch_pack_s(const SPlane& src, int storage, float* dst, int W, int H, int P,
                           cudaStream_t st);
@@ -111,12 +114,15 @@ cudaError_t launch_pd_consts(const LevelView& L, float lam, float eps, cudaStrea
 
 // Primal-dual iterations: n <= B iterations with halo B, tile variant
 // `variant`, state read from `in` and written to `out` (distinct buffers).
-// chained = true when the launch directly follows another k_pd launch on
-// the stream: it is then a programmatic dependent launch that loads its
-// per-warp constants while the preceding launch drains, and waits for it
-// before reading the state.
+// chained: PD_CHAINED (pd_tile.cuh) when the launch directly follows another
+// k_pd launch on the stream: it is then a programmatic dependent launch that
+// loads its per-warp constants while the preceding launch drains, and waits
+// for it before reading the state.  PD_CHAIN_START when it directly follows
+// the launch of this library that wrote the constants (launch_warp,
+// launch_clip_warp): a programmatic dependent launch too, which waits before
+// it reads anything.  0: an ordinary launch.
 cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const PDState& out,
-                      const PDParams& pp, int B, int n, cudaStream_t st, bool chained = false);
+                      const PDParams& pp, int B, int n, cudaStream_t st, int chained = 0);
 
 // The automatic schedule of `iters` iterations on a W x H level: a footprint
 // (variant), the number of launches and the halo depth (the iterations of
@@ -148,7 +154,7 @@ struct PdTmaMaps {
 // stall = 1 makes the first wait run out (testing aid).  Same results as
 // launch_pd.
 cudaError_t launch_pd_tma(const LevelView& L, const PDState& out, const PDParams& pp, int B,
-                          int n, bool chained, const PdTmaMaps& maps, int* status,
+                          int n, int chained, const PdTmaMaps& maps, int* status,
                           unsigned long long wait_ns, int stall, cudaStream_t st);
 // Dynamic shared memory of one k_pd_tma CTA for a storage type.
 size_t pd_tma_smem_bytes(int storage);

@@ -14,6 +14,7 @@
 
 #include "fs.h"
 #include "fs_kernels.h"
+#include "pd_tile.cuh"
 
 using namespace fs;
 
@@ -180,7 +181,7 @@ extern "C" fs_status fs_pd_iterate_noalloc(const float* d_I0, const unsigned cha
     int m = (iters - done) / (nl - k);
     if ((iters - done) % (nl - k)) ++m;
     e = launch_pd(ps.variant, L, (k % 2 == 0) ? A : Bs, (k % 2 == 0) ? Bs : A, pp, ps.depth, m,
-                  st, k > 0);
+                  st, k > 0 ? PD_CHAINED : 0);
     done += m;
   }
   if (e == cudaSuccess && nl % 2 == 1) {

@@ -262,13 +262,13 @@ __global__ void k_tensor(LevelView L, float beta, float eta, int precond) {
 // (launch_pd_consts' values: px_make of the stored sigma, tau, I_u, rho0
 // and u_w), written by the kernels that start a warp while they hold
 // I_u, rho0 and u_w.
-template <int S>
+template <int S, bool CG = false>
 __device__ __forceinline__ void pd_consts_px(const LevelView& L, size_t i, float Iu, float rho0,
                                              float uw, float lam, float eps) {
   PxRaw raw;
   raw.sx = raw.sy = 0.f;                     // not used by px_make's outputs below
-  raw.sig = L.sig[i];
-  raw.tau = L.tau[i];
+  raw.sig = ldf<CG>(L.sig + i);
+  raw.tau = ldf<CG>(L.tau + i);
   raw.Iu = round_storage<S>(Iu);
   raw.rho0 = round_storage<S>(rho0);
   raw.uw = uw;
@@ -301,14 +301,24 @@ __global__ void k_warp(LevelView L, int central, float lam, float eps, int const
 }
 
 // ------------------------------------------------------------ clip + update
+// CHAIN (k_clip_warp too): launched behind the warp's iterations as a
+// programmatic dependent launch.  The wait comes first, then the trigger that
+// lets the next launch be scheduled, and what those iterations or the last
+// warp start wrote is read through L2 (launches of a chain overlap, so an
+// SM's L1 may hold older lines).
+template <bool CHAIN>
 __global__ void k_clip(LevelView L, float du_max) {
+  if constexpr (CHAIN) {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+  }
   int x = blockIdx.x * blockDim.x + threadIdx.x;
   int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= L.W || y >= L.H) return;
   size_t i = (size_t)y * L.P + x;
   if (!(L.mask[i] & MASK_IN)) return;
   float2 w;
-  float un = clip_px<false>(L, i, du_max, w);
+  float un = clip_px<CHAIN>(L, i, du_max, w);
   L.u[i] = un;
   L.ubar[i] = un;
   L.uw[i] = un;
@@ -319,9 +329,13 @@ __global__ void k_clip(LevelView L, float du_max) {
 // k_warp at every pixel, with the updated w and u kept in registers (each
 // pixel's clip and linearisation read only that pixel's state; the gathers
 // read I1 and gamma', which neither writes).
-template <int S>
+template <int S, bool CHAIN>
 __global__ void k_clip_warp(LevelView L, float du_max, int central, float lam, float eps,
                             int consts) {
+  if constexpr (CHAIN) {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+  }
   int x = blockIdx.x * blockDim.x + threadIdx.x;
   int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= L.W || y >= L.H) return;
@@ -331,19 +345,19 @@ __global__ void k_clip_warp(LevelView L, float du_max, int central, float lam, f
   float u;
   if (L.mask[i] & MASK_IN) {
     float2 w;
-    u = clip_px<false>(L, i, du_max, w);
+    u = clip_px<CHAIN>(L, i, du_max, w);
     L.w[i] = w;
     L.u[i] = u;
     warp_px<S>(L, x, y, i, w, central, Iu, rho0, g);
   } else {
-    u = L.u[i];
+    u = ldf<CHAIN>(L.u + i);
   }
   sst<S>(L.Iu, i, Iu);
   sst<S>(L.rho0, i, rho0);
   L.g[i] = g;
   L.ubar[i] = u;
   L.uw[i] = u;
-  if (consts) pd_consts_px<S>(L, i, Iu, rho0, u, lam, eps);
+  if (consts) pd_consts_px<S, CHAIN>(L, i, Iu, rho0, u, lam, eps);
 }
 
 
@@ -440,6 +454,22 @@ __global__ void k_tensor_abc(LevelView L, float* __restrict__ dst) {
 namespace {
 dim3 grid_of(int W, int H) { return dim3((W + 31) / 32, (H + 7) / 8); }
 const dim3 kBlk(32, 8);
+
+// One thread per pixel of level L; chained: as a programmatic dependent
+// launch of the kernel before it on the stream.
+template <typename K, typename... A>
+cudaError_t launch_chained(K kernel, const LevelView& L, bool chained, cudaStream_t st, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid_of(L.W, L.H);
+  cfg.blockDim = kBlk;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, a...);
+}
 }  // namespace
 
 #define FS_STORAGE_SWITCH(st, CALL)                           \
@@ -489,9 +519,16 @@ cudaError_t launch_warp(const LevelView& L, int central, float lam, float eps, i
 }
 
 cudaError_t launch_clip_warp(const LevelView& L, float du_max, int central, float lam, float eps,
-                             int consts, cudaStream_t st) {
-  FS_STORAGE_SWITCH(L.st, (k_clip_warp<S><<<grid_of(L.W, L.H), kBlk, 0, st>>>(
-                              L, du_max, central, lam, eps, consts)))
+                             int consts, bool chained, cudaStream_t st) {
+  FS_STORAGE_SWITCH(L.st,
+                    return chained ? launch_chained(k_clip_warp<S, true>, L, true, st, L, du_max,
+                                                    central, lam, eps, consts)
+                                   : launch_chained(k_clip_warp<S, false>, L, false, st, L, du_max,
+                                                    central, lam, eps, consts))
+}
+cudaError_t launch_clip(const LevelView& L, float du_max, bool chained, cudaStream_t st) {
+  return chained ? launch_chained(k_clip<true>, L, true, st, L, du_max)
+                 : launch_chained(k_clip<false>, L, false, st, L, du_max);
 }
 cudaError_t launch_tensor_abc(const LevelView& L, float* dst, cudaStream_t st) {
   FS_STORAGE_SWITCH(L.st, (k_tensor_abc<S><<<grid_of(L.W, L.H), kBlk, 0, st>>>(L, dst)))

@@ -61,16 +61,16 @@ cudaError_t launch_pd_consts(const LevelView& L, float lam, float eps, cudaStrea
 }
 
 // MB: CTAs per SM the registers have to allow.
-template <int FW, int NY, int R, int S, bool ACC, int MB>
+template <int FW, int NY, int R, int S, bool ACC, int MB, bool CL2>
 __global__ void __launch_bounds__(FW * NY, MB)
 k_pd(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, int chained) {
   constexpr int FH = NY * R;
   __shared__ float s_ub[FH][FW];
   __shared__ float s_t1[FH][FW];
   __shared__ float s_t2[NY][FW];
-  pd_tile<FW, NY, R, S, ACC, false, true>(L, in, out, pp, B, n_iters, (int)blockIdx.x,
+  pd_tile<FW, NY, R, S, ACC, false, true, CL2>(L, in, out, pp, B, n_iters, (int)blockIdx.x,
                                           (int)blockIdx.y, (int)threadIdx.x, (int)threadIdx.y,
-                                          s_ub, s_t1, s_t2, chained != 0);
+                                          s_ub, s_t1, s_t2, chained);
 }
 
 template <int TW, int NY, int R, int S>
@@ -194,7 +194,7 @@ k_pd_cluster(LevelView L, PDParams pp, int n_iters) {
 
 template <int FW, int NY, int R, int S, bool ACC, int MB = (FW * NY >= 512 ? 1 : 2)>
 static cudaError_t launch_pd_t(const LevelView& L, const PDState& in, const PDState& out,
-                               const PDParams& pp, int B, int n, bool chained,
+                               const PDParams& pp, int B, int n, int chained,
                                cudaStream_t st) {
   const int IW = FW - 2 * B, IH = NY * R - 2 * B;
   if (IW <= 0 || IH <= 0 || n < 0 || n > B) return cudaErrorInvalidValue;
@@ -207,13 +207,17 @@ static cudaError_t launch_pd_t(const LevelView& L, const PDState& in, const PDSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_pd<FW, NY, R, S, ACC, MB>, L, in, out, pp, B, n, chained ? 1 : 0);
+  if (pp.fresh)
+    return cudaLaunchKernelEx(&cfg, k_pd<FW, NY, R, S, ACC, MB, true>, L, in, out, pp, B, n,
+                              chained);
+  return cudaLaunchKernelEx(&cfg, k_pd<FW, NY, R, S, ACC, MB, false>, L, in, out, pp, B, n,
+                            chained);
 }
 
 template <int S, bool ACC>
 static cudaError_t launch_pd_s(int variant, const LevelView& L, const PDState& in,
                                const PDState& out, const PDParams& pp, int B, int n,
-                               cudaStream_t st, bool chained) {
+                               cudaStream_t st, int chained) {
 #define FS_PD(...) return launch_pd_t<__VA_ARGS__>(L, in, out, pp, B, n, chained, st)
   switch (variant) {
     case PD_TILE_64: FS_PD(64, 8, 8, S, ACC);
@@ -301,7 +305,7 @@ PdSchedule pd_auto(int W, int H, int iters, int launches, int sms) {
 }
 
 cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const PDState& out,
-                      const PDParams& pp, int B, int n, cudaStream_t st, bool chained) {
+                      const PDParams& pp, int B, int n, cudaStream_t st, int chained) {
   if (pp.sched) {                       // the accelerated schedule: FP32 storage only
     if (L.st != ST_F32) return cudaErrorInvalidValue;
     return launch_pd_s<ST_F32, true>(variant, L, in, out, pp, B, n, st, chained);

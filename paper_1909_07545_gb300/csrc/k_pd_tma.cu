@@ -150,9 +150,9 @@ __device__ __forceinline__ float sval(const unsigned char* plane, int k) {
 
 // n_iters (<= B <= 8) iterations on every footprint of the level; the state
 // is read (through the copies in `maps`) from one buffer set and written to
-// `out`.  chained: a programmatic dependent launch (the first footprint's
-// constants are requested before the wait for the preceding launch, its
-// state after).  stall: testing aid, the first wait never completes.
+// `out`.  chained (pd_tile): PD_CHAINED requests the first footprint's
+// constants before the wait for the preceding launch and its state after,
+// PD_CHAIN_START waits first.  stall: testing aid, the first wait never completes.
 template <int S, bool ACC>
 __global__ void __launch_bounds__(kFW * kNY, 1)
 k_pd_tma(LevelView L, PDState out, PDParams pp, int B, int n_iters, int chained,
@@ -171,7 +171,9 @@ k_pd_tma(LevelView L, PDState out, PDParams pp, int B, int n_iters, int chained,
   const uint32_t bar = smem_addr(smem + Lay::bar);
 
   // the next launch of the chain may be scheduled once every CTA of this one
-  // is resident (it waits for this grid's completion before its state)
+  // is resident (it waits for this grid's completion before its state); for
+  // the first of a chain once the constants are complete
+  if (chained == PD_CHAIN_START) cudaGridDependencySynchronize();
   if (chained) cudaTriggerProgrammaticLaunchCompletion();
   int tile = blockIdx.x;
   if (leader) {
@@ -181,7 +183,7 @@ k_pd_tma(LevelView L, PDState out, PDParams pp, int B, int n_iters, int chained,
       request<S>(maps, smem, bar, tile, tiles_x, IH, B, true, false);
     }
   }
-  if (chained) cudaGridDependencySynchronize();
+  if (chained == PD_CHAINED) cudaGridDependencySynchronize();
   if (leader && tile < ntiles) request<S>(maps, smem, bar, tile, tiles_x, IH, B, false, true);
   __syncthreads();
 
@@ -272,7 +274,7 @@ namespace {
 
 template <int S, bool ACC>
 cudaError_t launch_tma_t(const LevelView& L, const PDState& out, const PDParams& pp, int B,
-                         int n, bool chained, const PdTmaMaps& maps, int* status,
+                         int n, int chained, const PdTmaMaps& maps, int* status,
                          unsigned long long wait_ns, int stall, cudaStream_t st) {
   using Lay = TmaLayout<S>;
   static bool configured = false;
@@ -300,7 +302,7 @@ cudaError_t launch_tma_t(const LevelView& L, const PDState& out, const PDParams&
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_pd_tma<S, ACC>, L, out, pp, B, n, chained ? 1 : 0, maps,
+  return cudaLaunchKernelEx(&cfg, k_pd_tma<S, ACC>, L, out, pp, B, n, chained, maps,
                             status, wait_ns, stall);
 }
 
@@ -315,7 +317,7 @@ size_t pd_tma_smem_bytes(int storage) {
 }
 
 cudaError_t launch_pd_tma(const LevelView& L, const PDState& out, const PDParams& pp, int B,
-                          int n, bool chained, const PdTmaMaps& maps, int* status,
+                          int n, int chained, const PdTmaMaps& maps, int* status,
                           unsigned long long wait_ns, int stall, cudaStream_t st) {
   if (B < 1 || B > kXM || n < 0 || n > B || L.W < 1 || L.H < 1) return cudaErrorInvalidValue;
   if (pp.sched) {

@@ -173,11 +173,11 @@ __device__ __noinline__ void pd_item(const PersistJob& J, const PersistPhase& ph
   if (J.variant == PD_TILE_64_T1024) {
     float(*s)[64] = reinterpret_cast<float(*)[64]>(smem);
     pd_tile<64, 16, 4, S, false, true>(L, in, out, J.pp, J.B, ph.n_iter, bx, by, t % 64, t / 64,
-                                       s, s + 64, s + 128, false);
+                                       s, s + 64, s + 128, 0);
   } else {
     float(*s)[32] = reinterpret_cast<float(*)[32]>(smem);
     pd_tile<32, 32, 1, S, false, true>(L, in, out, J.pp, J.B, ph.n_iter, bx, by, t % 32, t / 32,
-                                       s, s + 32, s + 64, false);
+                                       s, s + 32, s + 64, 0);
   }
 }
 

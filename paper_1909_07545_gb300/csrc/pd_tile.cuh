@@ -19,6 +19,9 @@
 
 namespace fs {
 
+// How a primal-dual launch follows the kernel before it (pd_tile).
+enum PdChain { PD_CHAINED = 1, PD_CHAIN_START = 2 };
+
 // The n_iters iterations of pd_tile on a thread's R rows (state in
 // registers, neighbours through shared memory); MASKED as in px_dual.
 template <int FW, int NY, int R, bool ACC, bool MASKED>
@@ -192,19 +195,24 @@ __device__ __forceinline__ void pd_iterate_rows(const PDParams& pp, int n_iters,
 // steps): iteration it of the block uses entry pp.k0 + it for sigma (all
 // pixels), tau and the L1 step (scaled from the stored tau_0 values, 0 off
 // the mask) and theta.  CG: the inputs may have been written by other CTAs
-// of the same launch (loads through L2 only).  chained: a programmatic
-// dependent launch of k_pd (constants loaded before the wait for the
-// preceding launch, the state after it).  s_ub, s_t1: shared arrays of
+// of the same launch (loads through L2 only).  chained: PD_CHAINED, a
+// programmatic dependent launch of k_pd behind another one (constants loaded
+// before the wait for it, the state after), PD_CHAIN_START, one behind the
+// kernel that wrote the constants (everything after the wait), or 0.  s_ub, s_t1: shared arrays of
 // FH x FW floats, s_t2 of NY x FW.  PRE: the per-warp constants are read
 // from L.dinv, L.sd, L.step, L.c0 (launch_pd_consts) instead of being
 // derived here from sigma, I_u, rho0 and u_w (the same bits either way).
-// Every thread of the CTA (FW x NY) must call it.
-template <int FW, int NY, int R, int S, bool ACC, bool CG, bool PRE = false>
+// CL2: the constants come through L2, for chains that start with
+// PD_CHAIN_START: no ordinary launch, at which an SM drops its L1's lines,
+// lies between the kernel that rewrote them and their reading.  (In long
+// chains behind an ordinary launch the L1 serves a tile's next launch on the
+// same SM, which is worth 4 % at 256 x 256.)  Every thread of the CTA (FW x NY) must call it.
+template <int FW, int NY, int R, int S, bool ACC, bool CG, bool PRE = false, bool CL2 = CG>
 __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
                                         const PDState& out, const PDParams& pp, int B,
                                         int n_iters, int bx, int by, int tx, int ty,
                                         float (*s_ub)[FW], float (*s_t1)[FW],
-                                        float (*s_t2)[FW], bool chained) {
+                                        float (*s_t2)[FW], int chained) {
   constexpr int FH = NY * R;
   const int IW = FW - 2 * B, IH = FH - 2 * B;
   const int ox = bx * IW - B;
@@ -215,7 +223,10 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
 
   // Let the next launch of the chain be scheduled as soon as every CTA of
   // this one is resident (it waits for this grid's completion before it
-  // reads the state, below).
+  // reads the state, below).  The first launch of a chain does so only once
+  // the constants are complete, which the next one reads without waiting.
+  if constexpr (CL2 && !CG)
+    if (chained == PD_CHAIN_START) cudaGridDependencySynchronize();
   if (chained) cudaTriggerProgrammaticLaunchCompletion();
 
   float u[R], ub[R], p1[R], p2[R];
@@ -240,8 +251,9 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
     for (int r = 0; r < R; ++r) {
       const unsigned i = idx[r];
       const float sx = sld_m<S, CG>(L.sx, i), sy = sld_m<S, CG>(L.sy, i);
-      const float tau = ldf<CG>(L.tau + i), dinv = ldf<CG>(L.dinv + i);
-      const float sd = ldf<CG>(L.sd + i), step = ldf<CG>(L.step + i), c0 = ldf<CG>(L.c0 + i);
+      const float tau = ldf<CG>(L.tau + i), dinv = ldf<CL2>(L.dinv + i);
+      const float sd = ldf<CL2>(L.sd + i), step = ldf<CL2>(L.step + i);
+      const float c0 = ldf<CL2>(L.c0 + i);
       const unsigned m8 = L.mask[i];
       // outside the level: the constants of all-zero inputs (px_make)
       c[r].sx = ok[r] ? sx : 0.f;
@@ -272,7 +284,11 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
   // (each triggers the next at its start), so an SM's L1 may hold lines of
   // this buffer set that the launch two before cached before it was
   // rewritten.
-  if (chained) cudaGridDependencySynchronize();
+  if constexpr (CL2 && !CG) {
+    if (chained == PD_CHAINED) cudaGridDependencySynchronize();
+  } else {
+    if (chained) cudaGridDependencySynchronize();
+  }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const float a = ldf<true>(in.u + idx[r]), b = ldf<true>(in.ubar + idx[r]);

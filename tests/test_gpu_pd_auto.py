@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 def _run(pair, choice, iters, **prm):
     s = make_solver(pair, levels=1, **prm)
     s.set_schedule([choice])
-    s.solve(pair["I0"], pair["I1"], 2, iters)
+    s.solve(pair["I0"], pair["I1"], 4, iters)
     out = [np64(s.read(0, b)) for b in ("U", "UBAR", "P")]
     s.close()
     return out
