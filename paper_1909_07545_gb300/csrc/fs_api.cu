@@ -67,6 +67,9 @@ struct HostLevel {
   int cluster = -1;                         // whole-level cluster variant, -1 if none
   int tuned = -1;                           // autotuned choice: 0 cluster, 1..8 depth, -1 none
   int tuned_variant = -1;                   // autotuned tile variant, -1: by size
+  // pd_auto's last answer and what it was asked (pd_plan)
+  mutable PdSchedule plan;
+  mutable int plan_iters = -1, plan_nl = -1;
   bool auto_best = false;                   // the tuner found pd_auto's schedule faster still
   LevelView v{};
   // tensor maps of the TMA-staged primal-dual footprints, reading buffer
@@ -450,14 +453,19 @@ PdSchedule pd_plan(const fs_handle* h, int l, int iters) {
   const int b = std::min(h->prm.block_iters, 8);
   if (b <= 0 && L.tuned >= 1 && !L.auto_best) {
     const int nl = pd_launch_count(iters, L.tuned);
-    return PdSchedule{L.tuned_variant, nl, (iters + nl - 1) / nl};
+    return PdSchedule{L.tuned_variant, nl, (iters + nl - 1) / nl, false};
   }
   int nl = 0;
   if (h->prm.storage != ST_F32)
     nl = pd_launch_count(iters, b > 0 ? b : (L.W > 512 || L.H > 512) ? 6 : 8);
   else if (b > 0 && (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0))
     nl = pd_launch_count(iters, b);
-  return pd_auto(L.W, L.H, iters, nl, h->sms);
+  if (L.plan_iters != iters || L.plan_nl != nl) {
+    L.plan = pd_auto(L.v, iters, nl, h->sms);
+    L.plan_iters = iters;
+    L.plan_nl = nl;
+  }
+  return L.plan;
 }
 
 // Whether a solve of h runs the TMA-staged footprints on some level.
@@ -561,6 +569,8 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
     const PDState& in = (k % 2 == 0) ? A : Bs;
     const PDState& out = (k % 2 == 0) ? Bs : A;
     pp.k0 = done;
+    pp.launches = nl;
+    pp.idle = !ps.skip ? -1 : k == 0 ? iters : 0;
     const int link = k > 0 ? PD_CHAINED : pp.fresh ? PD_CHAIN_START : 0;
     cudaError_t e = tma ? launch_pd_tma(L.v, out, pp, B, n, link, L.tma[k % 2], h->pd_status,
                                         h->wait_ns, (h->persist_stall && k == 0) ? 1 : 0, st)
@@ -1164,6 +1174,12 @@ fs_status fs_create(const fs_calib cam[2], const fs_pose* pose, int W, int H, in
     LevelView& v = L.v;
     v.W = L.W; v.H = L.H; v.P = L.P;
     v.st = p.storage;
+    // enlarged by 1e-4 of its radius, far more than the float rounding of the
+    // test against it
+    const double fr = 1.0001 * radial(cam[0], cam[0].fov_deg * M_PI / 360.0);
+    v.fov_cx = (float)L.cx; v.fov_cy = (float)L.cy;
+    v.fov_ix = (float)(1.0 / L.fx); v.fov_iy = (float)(1.0 / L.fy);
+    v.fov_r2 = (float)(fr * fr);
     v.mask = (const uint8_t*)take(plane8, l, "mask");
     float** fl[] = {&v.tau, &v.sig, &v.u, &v.ubar, &v.uw, &v.u_alt, &v.ubar_alt,
                     &v.dinv, &v.sd, &v.step, &v.c0};

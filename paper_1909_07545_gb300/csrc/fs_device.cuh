@@ -291,6 +291,14 @@ __device__ __forceinline__ void sst(const SPlane& pl, size_t i, float v) {
   else ((float*)pl.p)[i] = v;
 }
 
+// v as a plane of storage S holds it (rounded to nearest).
+template <int S>
+__device__ __forceinline__ float round_storage(float v) {
+  if constexpr (S == ST_F16) return __half2float(__float2half_rn(v));
+  else if constexpr (S == ST_BF16) return __bfloat162float(__float2bfloat16_rn(v));
+  else return v;
+}
+
 // Bilinear sample of a stored plane at (x + dx, y + dy), clamped.
 template <int S>
 __device__ __forceinline__ float sample_bilinear_s(const SPlane& img, int W, int H, int P, int x,
@@ -311,6 +319,9 @@ struct LevelView {
   int W, H, P;
   int st;                // Storage of the SPlane fields
   const uint8_t* mask;
+  // The FOV ellipse, slightly enlarged: every pixel of the mask has
+  // ((x - fov_cx) fov_ix)^2 + ((y - fov_cy) fov_iy)^2 <= fov_r2.
+  float fov_cx, fov_cy, fov_ix, fov_iy, fov_r2;
   SPlane I0, I1;
   float2* gamma;
   SPlane sx, sy;         // T^1/2 = I - s s^T, s = sqrt(1 - e) n  (Eq. 12)
@@ -353,6 +364,12 @@ struct PDParams {
   const float4* sched = nullptr;
   int k0 = 0;
   int fresh = 0;        // the chain of launches starts with PD_CHAIN_START
+  // Footprints without a pixel of the FOV (pd_tile): -1 = treated like the
+  // others; else left out, after `idle` iterations on their pixels in place
+  // (the warp's iterations at its first launch, 0 at the others).  Only on
+  // the footprints of pd_auto's `skip`.
+  int idle = -1;
+  int launches = 0;     // the warp's launches
 };
 
 }  // namespace fs

@@ -129,10 +129,14 @@ cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const 
 // the longest launch).  launches > 0 fixes the number of launches (16-bit
 // storage rounds the dual at each launch's end, so there it is part of the
 // result); 0 leaves it free.
+// skip: leave out the footprints without a FOV pixel (PDParams::idle).
+// L: the level's size and FOV ellipse (fov_r2 = infinity: every pixel may be
+// in the FOV).
 struct PdSchedule {
-  int variant, launches, depth;
+  int variant = 0, launches = 0, depth = 0;
+  bool skip = false;
 };
-PdSchedule pd_auto(int W, int H, int iters, int launches, int sms);
+PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms);
 // Launches of `iters` iterations at most `depth` each, made even when
 // iters >= 2 so that the ping-pong state ends where it began.
 int pd_launch_count(int iters, int depth);

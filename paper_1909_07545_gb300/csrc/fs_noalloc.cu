@@ -12,6 +12,8 @@
 #include <cstdio>
 #include <mutex>
 
+#include <cmath>
+
 #include "fs.h"
 #include "fs_kernels.h"
 #include "pd_tile.cuh"
@@ -149,6 +151,8 @@ extern "C" fs_status fs_pd_iterate_noalloc(const float* d_I0, const unsigned cha
   L.c0 = f + 12 * n;
   uint8_t* bits = (uint8_t*)(f + kFloatPlanes * n);
   L.mask = bits;
+  L.fov_r2 = INFINITY;               // any mask: no footprint is known to be outside
+  L.fov_ix = L.fov_iy = 1.f;
 
   // every scratch plane is written in full below before it is read, so the
   // contents left by an earlier call never reach this one
@@ -172,7 +176,7 @@ extern "C" fs_status fs_pd_iterate_noalloc(const float* d_I0, const unsigned cha
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const PdSchedule ps =
-      pd_auto(W, H, iters, p.block_iters > 0 ? pd_launch_count(iters, p.block_iters) : 0, sms);
+      pd_auto(L, iters, p.block_iters > 0 ? pd_launch_count(iters, p.block_iters) : 0, sms);
   const int nl = ps.launches;
   PDParams pp{p.lambda, p.huber_eps, p.theta};
   PDState A{L.u, L.ubar, L.p1, L.p2};

@@ -12,13 +12,6 @@ namespace fs {
 // A plane value in storage S (rounded to nearest) and, in lo, the part of
 // the float-float value v that the stored value leaves out.
 template <int S>
-__device__ __forceinline__ float round_storage(float v) {
-  if constexpr (S == ST_F16) return __half2float(__float2half_rn(v));
-  else if constexpr (S == ST_BF16) return __bfloat162float(__float2bfloat16_rn(v));
-  else return v;
-}
-
-template <int S>
 __device__ __forceinline__ void sst_df(const SPlane& pl, float* __restrict__ lo, size_t i, df v) {
   const float s = round_storage<S>(v.hi);
   sst<S>(pl, i, s);

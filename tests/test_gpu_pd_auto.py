@@ -43,3 +43,32 @@ def test_automatic_schedule_keeps_the_16_bit_rounding_points(W, H, iters, storag
     for a, b in zip(_run(p, -1, iters, storage=storage, pd_schedule=1),
                     _run(p, 24 + depth, iters, storage=storage, pd_schedule=1)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prm", [dict(), dict(precond=0, accel_gamma=0.3), dict(storage="f16"),
+                                 dict(storage="bf16", precond=0)])
+@pytest.mark.parametrize("W, H, iters", [(1100, 900, 12), (1100, 900, 31)])
+def test_footprints_outside_the_fov(W, H, iters, prm):
+    # a small FOV circle off the image's centre: most footprints hold no FOV
+    # pixel and are left out; the state outside the FOV, arbitrary here, still
+    # ends with the bits of the footprint that treats every pixel
+    cam = dict(model="equidistant", fx=120.0, fy=130.0, cx=400.3, cy=520.8, k=[0] * 4, fov_deg=170.0)
+    rng = np.random.default_rng(5)
+    p = dict(I0=rng.random((H, W)), I1=rng.random((H, W)), cam0=cam, cam1=dict(cam), R=np.eye(3),
+             t=np.array([-0.1, 0.0, 0.0]), levels=1)
+    state = {"U": rng.uniform(-1, 1, (H, W)), "UBAR": rng.uniform(-1, 1, (H, W)),
+             "P": rng.uniform(-0.9, 0.9, (2, H, W))}
+    outs = []
+    for choice in (-1, 30):                           # 30: depth 6 on 64 x 64
+        s = make_solver(p, levels=1, **prm)
+        s.set_schedule([choice])
+        s.solve(p["I0"], p["I1"], 1, 2)
+        for b, v in state.items():
+            s.write(0, b, v)
+        s.stage(0, "PD", iters)
+        outs.append([np64(s.read(0, b)) for b in state])
+        s.solve(p["I0"], p["I1"], 2, iters)
+        outs[-1] += [np64(s.read(0, b)) for b in state]
+        s.close()
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
