@@ -116,7 +116,7 @@ typedef struct {
  * TGV-L1 energy of Eq. 10, lambda |rho| + alpha1 |T^1/2 grad u - v| +
  * alpha0 |grad v| (alpha0 = 17, alpha1 = 1.2 in Sec. IV-C; huber_eps and
  * pd_schedule do not apply; block_iters is the temporal-blocking depth, 0 =
- * tuned or 4), solved by the primal-dual steps of Eq. 11 with diagonal
+ * tuned, or chosen by level size), solved by the primal-dual steps of Eq. 11 with diagonal
  * preconditioning; FP32 storage only.
  * deriv: how I_u, the derivative of the warped I1 along the trajectory, is
  * taken.  FS_DERIV_FORWARD (0) = I1(x + w + g) - I1(x + w), the difference of

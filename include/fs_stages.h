@@ -118,7 +118,7 @@ fs_status fs_timing_read(fs_handle* h, double* ms, long long* launches,
  * candidates are 0 = a dual and a primal launch per iteration and 8 v + d =
  * temporal-blocking depth d on a 32 x 32 footprint of 256 (v = 0, choices
  * 1..8), 1024 (v = 1, 9..16) or 512 threads (v = 2, 17..24), or a 64 x 32
- * footprint of 512 (v = 3, 25..32) or 1024 threads (v = 4, 33..40).  Each Huber-TV level is timed
+ * footprint of 512 (v = 3, 25..32) or 1024 threads (v = 4, 33..40).  Each level is timed
  * once more in the automatic schedule, whose footprints and depths go beyond
  * this encoding: where that is faster, the handle keeps it and choice reports
  * the fastest encoded one.  Overwrites the levels' state; synchronises the

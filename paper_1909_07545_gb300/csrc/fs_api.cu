@@ -444,24 +444,28 @@ bool use_cluster(const fs_handle* h, int l) {
 }
 
 // The temporal-blocking launches of `iters` iterations on level l: the tuned
-// choice, else pd_auto.  block_iters, when set, fixes the number of
+// choice (TGV: 0 launches = a launch per step), else pd_auto or tgv_auto.  block_iters, when set, fixes the number of
 // launches, and so does 16-bit storage (depth 6 on levels wider than 512 px,
 // 8 below), whose results depend on it.  A halo is never deeper than the
 // longest launch's iterations.
 PdSchedule pd_plan(const fs_handle* h, int l, int iters) {
   const HostLevel& L = h->lv[l];
   const int b = std::min(h->prm.block_iters, 8);
+  const bool tgv = h->prm.regularizer == FS_REG_TGV;
+  if (tgv && b <= 0 && L.tuned == 0 && !L.auto_best) return PdSchedule{};
   if (b <= 0 && L.tuned >= 1 && !L.auto_best) {
     const int nl = pd_launch_count(iters, L.tuned);
     return PdSchedule{L.tuned_variant, nl, (iters + nl - 1) / nl, false};
   }
   int nl = 0;
-  if (h->prm.storage != ST_F32)
+  if (tgv)
+    nl = b > 0 ? pd_launch_count(iters, b) : 0;
+  else if (h->prm.storage != ST_F32)
     nl = pd_launch_count(iters, b > 0 ? b : (L.W > 512 || L.H > 512) ? 6 : 8);
   else if (b > 0 && (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0))
     nl = pd_launch_count(iters, b);
   if (L.plan_iters != iters || L.plan_nl != nl) {
-    L.plan = pd_auto(L.v, iters, nl, h->sms);
+    L.plan = tgv ? tgv_auto(L.v, iters, nl, h->sms) : pd_auto(L.v, iters, nl, h->sms);
     L.plan_iters = iters;
     L.plan_nl = nl;
   }
@@ -539,11 +543,7 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
   }
   if (h->prm.regularizer == FS_REG_TGV) {
     TgvParams tp{h->prm.lambda, h->prm.theta, h->prm.alpha0, h->prm.alpha1, h->prm.precond};
-    // block_iters when set, else the tuned depth, else 4 (0 = launch per
-    // step); the tuned footprint, else the 256-thread one
-    int B = h->prm.block_iters > 0 ? h->prm.block_iters : (L.tuned >= 0 ? L.tuned : 4);
-    int v = (h->prm.block_iters <= 0 && L.tuned_variant >= 0) ? L.tuned_variant : 0;
-    FS_LAUNCH("k_tgv", launch_tgv_iterations(L.v, tp, B, v, iters, st));
+    FS_LAUNCH("k_tgv", launch_tgv_iterations(L.v, tp, pd_plan(h, l, iters), iters, st));
     return FS_OK;
   }
   if (use_cluster(h, l)) {
@@ -2040,7 +2040,7 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
     // encoding: where it is faster still, the handle keeps it and `choice`
     // reports the best encoded one
     bool auto_best = false;
-    if (h->prm.regularizer != FS_REG_TGV && saved_block <= 0 && st == FS_OK) {
+    if (saved_block <= 0 && st == FS_OK) {
       h->prm.pd_schedule = saved_sched == 0 ? 0 : 1;
       L.tuned = L.tuned_variant = -1;
       auto_best = time_level() < best;

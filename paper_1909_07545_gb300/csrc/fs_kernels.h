@@ -70,14 +70,42 @@ cudaError_t launch_zero_state(const LevelView& L, cudaStream_t st);
 cudaError_t launch_warm_start(const LevelView& L, float du_max, cudaStream_t st);
 cudaError_t launch_continue(const LevelView& L, cudaStream_t st);
 
-// TGV-L1 (k_tgv.cu): n iterations, with B = 0 as a dual and a primal launch
-// each, else temporally blocked with at most B (1..8) per launch on 32 x 32
-// footprints of 256 (variant 0), 1024 (1) or 512 (2) threads, or 64 x 32
-// footprints of 512 (3) or 1024 (4) threads (identical results); v, vbar,
-// q <- 0; vbar <- v at a warp's start.
+// The automatic schedule of `iters` iterations on a level: a footprint
+// (variant), the number of launches and the halo depth (the iterations of
+// the longest launch).  launches > 0 fixes the number of launches (16-bit
+// storage rounds the dual at each launch's end, so there it is part of the
+// result); 0 leaves it free.  skip: leave out the footprints without a FOV
+// pixel (PDParams::idle).  L: the level's size and FOV ellipse (fov_r2 =
+// infinity: every pixel may be in the FOV).
+struct PdSchedule {
+  int variant = 0, launches = 0, depth = 0;
+  bool skip = false;
+};
+// A footprint the rule may pick: fw x fh pixels, per_sm of them on an SM at
+// once; a launch of n iterations takes t0 + n b microseconds per wave of
+// them; skip: instantiated without the footprints outside the FOV.
+struct BlockFit {
+  int variant, fw, fh, per_sm;
+  float t0, b;
+  bool skip;
+};
+// The least of the modelled times over n_fit footprints and launch counts.
+PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, int iters,
+                          int launches, int sms);
+PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms);    // Huber-TV
+PdSchedule tgv_auto(const LevelView& L, int iters, int launches, int sms);   // TGV-L1
+// Launches of `iters` iterations at most `depth` each, made even when
+// iters >= 2 so that the ping-pong state ends where it began.
+int pd_launch_count(int iters, int depth);
+
+// TGV-L1 (k_tgv.cu): n iterations, with ps.launches = 0 as a dual and a
+// primal launch each, else temporally blocked on the footprint ps.variant --
+// 0..4, the encoding of fs_autotune: 32 x 32 of 256 (variant 0), 1024 (1) or
+// 512 (2) threads, 64 x 32 of 512 (3) or 1024 (4) threads; further ones of
+// tgv_auto (identical results); v, vbar, q <- 0; vbar <- v at a warp's start.
 constexpr int kTgvVariants = 5;
 struct TgvParams;
-cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, int B, int variant,
+cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, const PdSchedule& ps,
                                   int n, cudaStream_t st);
 cudaError_t launch_tgv_reset(const LevelView& L, cudaStream_t st);
 // Energy terms of a level summed into acc[0..2] (data, regulariser, L1
@@ -123,23 +151,6 @@ cudaError_t launch_pd_consts(const LevelView& L, float lam, float eps, cudaStrea
 // it reads anything.  0: an ordinary launch.
 cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const PDState& out,
                       const PDParams& pp, int B, int n, cudaStream_t st, int chained = 0);
-
-// The automatic schedule of `iters` iterations on a W x H level: a footprint
-// (variant), the number of launches and the halo depth (the iterations of
-// the longest launch).  launches > 0 fixes the number of launches (16-bit
-// storage rounds the dual at each launch's end, so there it is part of the
-// result); 0 leaves it free.
-// skip: leave out the footprints without a FOV pixel (PDParams::idle).
-// L: the level's size and FOV ellipse (fov_r2 = infinity: every pixel may be
-// in the FOV).
-struct PdSchedule {
-  int variant = 0, launches = 0, depth = 0;
-  bool skip = false;
-};
-PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms);
-// Launches of `iters` iterations at most `depth` each, made even when
-// iters >= 2 so that the ping-pong state ends where it began.
-int pd_launch_count(int iters, int depth);
 
 // The tensor maps k_pd_tma copies a footprint through: T^1/2, tau, the
 // per-warp constants (launch_pd_consts) and the mask of a level, and the

@@ -254,11 +254,8 @@ int pd_launch_count(int iters, int depth) {
   return n;
 }
 
-// The least of the modelled times over footprints and launch counts.  A
-// launch of n iterations takes t0 + n b microseconds per wave of CTAs (per_sm
-// of them on every SM): t0 the launch, the loads and the stores, b one
-// iteration, both fitted to the sizes of the table below on GB300 (graph
-// replays, warm).  What the rule picks against the fixed choice it replaces
+// t0: the launch, the loads and the stores, b: one iteration, both fitted to
+// the sizes of the table below on GB300 (graph replays, warm).  What the rule picks against the fixed choice it replaces
 // (64 x 64 footprints of 512 threads at depth 8, at depth 6 above 512 pixels,
 // 32 x 32 of 256 threads below 128), us per 10 / 100 iterations:
 //   64 x 64     5.8 / 39.4   against   7.4 / 49.2
@@ -272,12 +269,7 @@ int pd_launch_count(int iters, int depth) {
 // 2048 frame under a 180-degree lens takes 24.0 ms against 27.9.  (With a
 // single wave the test only costs, up to 4 % of a 256 x 256 frame.)
 PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms) {
-  struct Fit {
-    int variant, fw, fh, per_sm;
-    float t0, b;
-    bool skip;                 // instantiated without the footprints outside the FOV
-  };
-  static const Fit kFit[] = {
+  static const BlockFit kFit[] = {
       {PD_TILE_32x16_T256, 32, 16, 1, 1.95f, 0.18f, false},
       {PD_TILE_32x24_T384, 32, 24, 1, 1.85f, 0.185f, false},
       {PD_TILE_32_T512, 32, 32, 1, 1.7f, 0.245f, false},
@@ -289,15 +281,20 @@ PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms) {
       {PD_TILE_64_T1024, 64, 64, 1, 4.1f, 0.735f, true},
       {PD_TILE_64x32_T512, 64, 32, 2, 3.2f, 0.67f, true},
   };
+  return block_schedule(kFit, (int)(sizeof(kFit) / sizeof(kFit[0])), L, iters, launches, sms);
+}
+
+PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, int iters,
+                          int launches, int sms) {
   constexpr int kMaxDepth = 15;
   PdSchedule best;
-  best.variant = PD_TILE_32_T512;
   best.launches = launches > 0 ? launches : pd_launch_count(iters, 8);
   double best_us = 1e300;
   auto consider = [&](int nl) {
     const int depth = std::max(1, (iters + nl - 1) / nl);
     if (depth > kMaxDepth) return;
-    for (const Fit& f : kFit) {
+    for (int j = 0; j < n_fit; ++j) {
+      const BlockFit& f = fit[j];
       const int iw = f.fw - 2 * depth, ih = f.fh - 2 * depth;
       if (iw < 2 || ih < 2) continue;
       const int tx = (L.W + iw - 1) / iw, ty = (L.H + ih - 1) / ih;

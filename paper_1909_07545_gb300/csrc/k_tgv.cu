@@ -26,6 +26,7 @@
 
 #include "fs_kernels.h"
 #include "pd_tgv_math.cuh"
+#include "pd_tile.cuh"
 
 namespace fs {
 
@@ -116,26 +117,216 @@ struct TgvState {
   float* s[12];   // u, ubar, v1, v2, vb1, vb2, p1, p2, q11, q12, q21, q22
 };
 
-// FTZ as in tgv_ball.
-template <int FW, int NY, int R, bool FTZ>
-__global__ void __launch_bounds__(FW * NY, FW * NY >= 512 ? 1 : 2)
-k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n_iters,
-              int chained) {
+// Shared memory of a footprint: what neighbours read of each other.  ubar,
+// vbar (the dual reads them from the right and from below) and t1, qx (the
+// primal reads them from the left) for every pixel; t2, qy (read from above)
+// only for the last row of each thread, as a thread keeps its other rows.
+template <int FW, int NY, int R>
+struct TgvShared {
+  float ub[NY * R][FW], vb1[NY * R][FW], vb2[NY * R][FW];
+  float t1[NY * R][FW], qx1[NY * R][FW], qx2[NY * R][FW];
+  float t2[NY][FW], qy1[NY][FW], qy2[NY][FW];
+};
+
+// A thread's R rows: u, ubar, v, vbar, p, q.
+template <int R>
+struct TgvRows {
+  float u[R], ub[R], v1[R], v2[R], vb1[R], vb2[R], p1[R], p2[R], q11[R], q12[R], q21[R], q22[R];
+};
+
+// n_iters iterations on a thread's rows (neighbours through sm); FTZ as in
+// tgv_ball, MASKED as in tgv_px_dual.  Rows in pairs (j, j + H) on the packed
+// FP32 operations, as in pd_iterate2: the rows below pair j are pair j + 1,
+// those above it pair j - 1; the same values in the same order, so the same
+// bits.
+template <int FW, int NY, int R, bool FTZ, bool MASKED>
+__device__ __forceinline__ void tgv_iterate(const TgvParams& tp, int n_iters, int tx, int ty,
+                                            unsigned mb, const TgvConst (&c)[R], TgvRows<R>& s,
+                                            TgvShared<FW, NY, R>& sm) {
   constexpr int FH = NY * R;
-  // neighbours' values: ubar, vbar (read by the dual from the right / below)
-  // and t, masked q (read by the primal from the left / above); nine FH x FW
-  // planes of dynamic shared memory (tgv_smem_bytes)
+  const int txr = min(tx + 1, FW - 1), txl = max(tx - 1, 0);
+  const int fnext = min(ty * R + R, FH - 1);     // the thread below's first row
+  if constexpr (R % 2 == 0) {
+    constexpr int H = R / 2;
+    TgvConst2 c2[H];
+    float2 u2[H], ub2[H], v12[H], v22[H], vb12[H], vb22[H], p12[H], p22[H];
+    float2 q112[H], q122[H], q212[H], q222[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      c2[j] = tgv_pair(c[j], c[j + H]);
+      u2[j] = make_float2(s.u[j], s.u[j + H]);
+      ub2[j] = make_float2(s.ub[j], s.ub[j + H]);
+      v12[j] = make_float2(s.v1[j], s.v1[j + H]);
+      v22[j] = make_float2(s.v2[j], s.v2[j + H]);
+      vb12[j] = make_float2(s.vb1[j], s.vb1[j + H]);
+      vb22[j] = make_float2(s.vb2[j], s.vb2[j + H]);
+      p12[j] = make_float2(s.p1[j], s.p1[j + H]);
+      p22[j] = make_float2(s.p2[j], s.p2[j + H]);
+      q112[j] = make_float2(s.q11[j], s.q11[j + H]);
+      q122[j] = make_float2(s.q12[j], s.q12[j + H]);
+      q212[j] = make_float2(s.q21[j], s.q21[j + H]);
+      q222[j] = make_float2(s.q22[j], s.q22[j + H]);
+    }
+    const float2 th2 = make_float2(tp.theta, tp.theta);
+    float2 t12[H], t22[H], qx12[H], qx22[H], qy12[H], qy22[H];
+#pragma unroll 1
+    for (int it = 0; it < n_iters; ++it) {
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        const int f0 = ty * R + j, f1 = f0 + H;
+        const bool last = j + 1 == H;
+        const int k = last ? j : j + 1;
+        const float2 ub_b = last ? make_float2(ub2[0].y, sm.ub[fnext][tx]) : ub2[k];
+        const float2 vb1_b = last ? make_float2(vb12[0].y, sm.vb1[fnext][tx]) : vb12[k];
+        const float2 vb2_b = last ? make_float2(vb22[0].y, sm.vb2[fnext][tx]) : vb22[k];
+        tgv_px_dual2<FTZ, MASKED>(
+            mb >> (3 * j), mb >> (3 * (j + H)), ub2[j],
+            make_float2(sm.ub[f0][txr], sm.ub[f1][txr]), ub_b, vb12[j],
+            make_float2(sm.vb1[f0][txr], sm.vb1[f1][txr]), vb1_b, vb22[j],
+            make_float2(sm.vb2[f0][txr], sm.vb2[f1][txr]), vb2_b, c2[j], tp, p12[j], p22[j],
+            q112[j], q122[j], q212[j], q222[j], t12[j], t22[j], qx12[j], qx22[j], qy12[j],
+            qy22[j]);
+        sm.t1[f0][tx] = t12[j].x;   sm.t1[f1][tx] = t12[j].y;
+        sm.qx1[f0][tx] = qx12[j].x; sm.qx1[f1][tx] = qx12[j].y;
+        sm.qx2[f0][tx] = qx22[j].x; sm.qx2[f1][tx] = qx22[j].y;
+        if (last) {                                    // row R - 1
+          sm.t2[ty][tx] = t22[j].y;
+          sm.qy1[ty][tx] = qy12[j].y;
+          sm.qy2[ty][tx] = qy22[j].y;
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < H; ++j) {
+        const int f0 = ty * R + j, f1 = f0 + H;
+        // above: the previous pair, or for the first pair the thread above's
+        // last row (the footprint's top row, halo, reads its own) and row H - 1
+        float2 t2_u, qy1_u, qy2_u;
+        if (j > 0) {
+          t2_u = t22[j > 0 ? j - 1 : 0];
+          qy1_u = qy12[j > 0 ? j - 1 : 0];
+          qy2_u = qy22[j > 0 ? j - 1 : 0];
+        } else {
+          t2_u = make_float2(ty > 0 ? sm.t2[ty - 1][tx] : t22[0].x, t22[H - 1].x);
+          qy1_u = make_float2(ty > 0 ? sm.qy1[ty - 1][tx] : qy12[0].x, qy12[H - 1].x);
+          qy2_u = make_float2(ty > 0 ? sm.qy2[ty - 1][tx] : qy22[0].x, qy22[H - 1].x);
+        }
+        tgv_px_primal2(t12[j], make_float2(sm.t1[f0][txl], sm.t1[f1][txl]), t22[j], t2_u,
+                       qx12[j], make_float2(sm.qx1[f0][txl], sm.qx1[f1][txl]), qy12[j], qy1_u,
+                       qx22[j], make_float2(sm.qx2[f0][txl], sm.qx2[f1][txl]), qy22[j], qy2_u,
+                       p12[j], p22[j], c2[j], th2, u2[j], ub2[j], v12[j], v22[j], vb12[j],
+                       vb22[j]);
+        sm.ub[f0][tx] = ub2[j].x;   sm.ub[f1][tx] = ub2[j].y;
+        sm.vb1[f0][tx] = vb12[j].x; sm.vb1[f1][tx] = vb12[j].y;
+        sm.vb2[f0][tx] = vb22[j].x; sm.vb2[f1][tx] = vb22[j].y;
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      s.u[j] = u2[j].x;     s.u[j + H] = u2[j].y;
+      s.ub[j] = ub2[j].x;   s.ub[j + H] = ub2[j].y;
+      s.v1[j] = v12[j].x;   s.v1[j + H] = v12[j].y;
+      s.v2[j] = v22[j].x;   s.v2[j + H] = v22[j].y;
+      s.vb1[j] = vb12[j].x; s.vb1[j + H] = vb12[j].y;
+      s.vb2[j] = vb22[j].x; s.vb2[j + H] = vb22[j].y;
+      s.p1[j] = p12[j].x;   s.p1[j + H] = p12[j].y;
+      s.p2[j] = p22[j].x;   s.p2[j + H] = p22[j].y;
+      s.q11[j] = q112[j].x; s.q11[j + H] = q112[j].y;
+      s.q12[j] = q122[j].x; s.q12[j + H] = q122[j].y;
+      s.q21[j] = q212[j].x; s.q21[j + H] = q212[j].y;
+      s.q22[j] = q222[j].x; s.q22[j + H] = q222[j].y;
+    }
+  } else {
+    float t1[R], t2[R], qx1[R], qx2[R], qy1[R], qy2[R];
+#pragma unroll 1
+    for (int it = 0; it < n_iters; ++it) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int fy = ty * R + r;
+        const int k = r + 1 < R ? r + 1 : r;
+        const float ub_b = (r + 1 < R) ? s.ub[k] : sm.ub[fnext][tx];
+        const float vb1_b = (r + 1 < R) ? s.vb1[k] : sm.vb1[fnext][tx];
+        const float vb2_b = (r + 1 < R) ? s.vb2[k] : sm.vb2[fnext][tx];
+        tgv_px_dual<FTZ, MASKED>(mb >> (3 * r), s.ub[r], sm.ub[fy][txr], ub_b, s.vb1[r],
+                                 sm.vb1[fy][txr], vb1_b, s.vb2[r], sm.vb2[fy][txr], vb2_b, c[r],
+                                 tp, s.p1[r], s.p2[r], s.q11[r], s.q12[r], s.q21[r], s.q22[r],
+                                 t1[r], t2[r], qx1[r], qx2[r], qy1[r], qy2[r]);
+        sm.t1[fy][tx] = t1[r];
+        sm.qx1[fy][tx] = qx1[r];
+        sm.qx2[fy][tx] = qx2[r];
+        if (r + 1 == R) {
+          sm.t2[ty][tx] = t2[r];
+          sm.qy1[ty][tx] = qy1[r];
+          sm.qy2[ty][tx] = qy2[r];
+        }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int fy = ty * R + r;
+        const int k = r > 0 ? r - 1 : 0;
+        const float t2_u = r > 0 ? t2[k] : (ty > 0 ? sm.t2[ty - 1][tx] : t2[0]);
+        const float qy1_u = r > 0 ? qy1[k] : (ty > 0 ? sm.qy1[ty - 1][tx] : qy1[0]);
+        const float qy2_u = r > 0 ? qy2[k] : (ty > 0 ? sm.qy2[ty - 1][tx] : qy2[0]);
+        tgv_px_primal(t1[r], sm.t1[fy][txl], t2[r], t2_u, qx1[r], sm.qx1[fy][txl], qy1[r], qy1_u,
+                      qx2[r], sm.qx2[fy][txl], qy2[r], qy2_u, s.p1[r], s.p2[r], c[r], tp.theta,
+                      s.u[r], s.ub[r], s.v1[r], s.v2[r], s.vb1[r], s.vb2[r]);
+        sm.ub[fy][tx] = s.ub[r];
+        sm.vb1[fy][tx] = s.vb1[r];
+        sm.vb2[fy][tx] = s.vb2[r];
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// n iterations, in place, on the interior pixels of a footprint without a FOV
+// pixel: they move on their own (every step size is 0 there), and not at all
+// where p = q = 0, ubar = u and vbar = v, as every warp of a solve starts.
+template <int FW, int NY, int R, bool FTZ>
+__device__ __forceinline__ void tgv_idle(const LevelView& L, const TgvState& io,
+                                         const TgvParams& tp, int B, int n, int ox, int oy,
+                                         int tx, int ty) {
+  const int gx = ox + tx;
+  if (gx < 0 || gx >= L.W || tx < B || tx >= FW - B) return;
+#pragma unroll 1
+  for (int r = 0; r < R; ++r) {
+    const int fy = ty * R + r, gy = oy + fy;
+    if (gy < 0 || gy >= L.H || fy < B || fy >= NY * R - B) continue;
+    const size_t i = (size_t)gy * L.P + gx;
+    float a[12];
+    bool rest = true;
+#pragma unroll
+    for (int j = 0; j < 12; ++j) a[j] = __ldcg(io.s[j] + i);
+#pragma unroll
+    for (int j = 6; j < 12; ++j) rest = rest && a[j] == 0.f;
+    if (rest && a[0] == a[1] && a[2] == a[4] && a[3] == a[5]) continue;
+    TgvConst c;
+    tgv_const(0u, 0u, 0u, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, tp, c);
+    for (int it = 0; it < n; ++it) {
+      float t1, t2, x1, x2, y1, y2;
+      tgv_px_dual<FTZ>(0u, a[1], 0.f, 0.f, a[4], 0.f, 0.f, a[5], 0.f, 0.f, c, tp, a[6], a[7],
+                       a[8], a[9], a[10], a[11], t1, t2, x1, x2, y1, y2);
+      tgv_px_primal(t1, 0.f, t2, 0.f, x1, 0.f, y1, 0.f, x2, 0.f, y2, 0.f, a[6], a[7], c, tp.theta,
+                    a[0], a[1], a[2], a[3], a[4], a[5]);
+    }
+#pragma unroll
+    for (int j = 0; j < 12; ++j) io.s[j][i] = a[j];
+  }
+}
+
+// One launch of n_iters <= B iterations on FW x (NY R) footprints with halo
+// B; MB: CTAs per SM the registers have to allow.  IDLE: footprints without
+// a FOV pixel are left out, after `idle` iterations on their pixels in place
+// (the warp's iterations at its first launch, 0 at the others).
+template <int FW, int NY, int R, int MB, bool FTZ, bool IDLE>
+__global__ void __launch_bounds__(FW * NY, MB)
+k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n_iters,
+              int chained, int idle) {
+  constexpr int FH = NY * R;
   extern __shared__ float tgv_smem[];
-  typedef float Plane[FW];
-  Plane* s_ub = reinterpret_cast<Plane*>(tgv_smem + 0 * FH * FW);
-  Plane* s_vb1 = reinterpret_cast<Plane*>(tgv_smem + 1 * FH * FW);
-  Plane* s_vb2 = reinterpret_cast<Plane*>(tgv_smem + 2 * FH * FW);
-  Plane* s_t1 = reinterpret_cast<Plane*>(tgv_smem + 3 * FH * FW);
-  Plane* s_t2 = reinterpret_cast<Plane*>(tgv_smem + 4 * FH * FW);
-  Plane* s_qx1 = reinterpret_cast<Plane*>(tgv_smem + 5 * FH * FW);
-  Plane* s_qx2 = reinterpret_cast<Plane*>(tgv_smem + 6 * FH * FW);
-  Plane* s_qy1 = reinterpret_cast<Plane*>(tgv_smem + 7 * FH * FW);
-  Plane* s_qy2 = reinterpret_cast<Plane*>(tgv_smem + 8 * FH * FW);
+  TgvShared<FW, NY, R>& sm = *reinterpret_cast<TgvShared<FW, NY, R>*>(tgv_smem);
 
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int IW = FW - 2 * B, IH = FH - 2 * B;
@@ -144,6 +335,13 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
   const int gx = ox + tx;
   const bool col_in = gx >= 0 && gx < L.W;
 
+  if constexpr (IDLE) {              // as in pd_tile
+    if (outside_fov(L, ox, oy, FW, FH)) {
+      if (chained && blockIdx.x == 0 && blockIdx.y == 0) cudaGridDependencySynchronize();
+      if (idle > 0) tgv_idle<FW, NY, R, FTZ>(L, in, tp, B, idle, ox, oy, tx, ty);
+      return;
+    }
+  }
   if (chained) cudaTriggerProgrammaticLaunchCompletion();
 
   // constants (written before the chain; unconditional loads from clamped
@@ -191,8 +389,7 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
   // launch may start while the launch two before it still caches lines of
   // this buffer set in L1)
   if (chained) cudaGridDependencySynchronize();
-  float u[R], ub[R], v1[R], v2[R], vb1[R], vb2[R], p1[R], p2[R], q11[R], q12[R], q21[R],
-      q22[R];
+  TgvRows<R> s;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const unsigned k = idx[r];
@@ -200,141 +397,21 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
 #pragma unroll
     for (int j = 0; j < 12; ++j) a[j] = __ldcg(in.s[j] + k);
     const float z = ok[r] ? 1.f : 0.f;   // off the level: inert zeros
-    u[r] = a[0] * z; ub[r] = a[1] * z; v1[r] = a[2] * z; v2[r] = a[3] * z;
-    vb1[r] = a[4] * z; vb2[r] = a[5] * z; p1[r] = a[6] * z; p2[r] = a[7] * z;
-    q11[r] = a[8] * z; q12[r] = a[9] * z; q21[r] = a[10] * z; q22[r] = a[11] * z;
+    s.u[r] = a[0] * z; s.ub[r] = a[1] * z; s.v1[r] = a[2] * z; s.v2[r] = a[3] * z;
+    s.vb1[r] = a[4] * z; s.vb2[r] = a[5] * z; s.p1[r] = a[6] * z; s.p2[r] = a[7] * z;
+    s.q11[r] = a[8] * z; s.q12[r] = a[9] * z; s.q21[r] = a[10] * z; s.q22[r] = a[11] * z;
     const int fy = ty * R + r;
-    s_ub[fy][tx] = ub[r];
-    s_vb1[fy][tx] = vb1[r];
-    s_vb2[fy][tx] = vb2[r];
+    sm.ub[fy][tx] = s.ub[r];
+    sm.vb1[fy][tx] = s.vb1[r];
+    sm.vb2[fy][tx] = s.vb2[r];
   }
-  __syncthreads();
-
-  const int txr = min(tx + 1, FW - 1), txl = max(tx - 1, 0);
-  if constexpr (R % 2 == 0) {
-    // rows in pairs (j, j + H) on the packed FP32 operations, as in
-    // pd_iterate2: the rows below pair j are pair j + 1, those above it
-    // pair j - 1; the same values in the same order, so the same bits
-    constexpr int H = R / 2;
-    TgvConst2 c2[H];
-    float2 u2[H], ub2[H], v12[H], v22[H], vb12[H], vb22[H], p12[H], p22[H];
-    float2 q112[H], q122[H], q212[H], q222[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      c2[j] = tgv_pair(c[j], c[j + H]);
-      u2[j] = make_float2(u[j], u[j + H]);
-      ub2[j] = make_float2(ub[j], ub[j + H]);
-      v12[j] = make_float2(v1[j], v1[j + H]);
-      v22[j] = make_float2(v2[j], v2[j + H]);
-      vb12[j] = make_float2(vb1[j], vb1[j + H]);
-      vb22[j] = make_float2(vb2[j], vb2[j + H]);
-      p12[j] = make_float2(p1[j], p1[j + H]);
-      p22[j] = make_float2(p2[j], p2[j + H]);
-      q112[j] = make_float2(q11[j], q11[j + H]);
-      q122[j] = make_float2(q12[j], q12[j + H]);
-      q212[j] = make_float2(q21[j], q21[j + H]);
-      q222[j] = make_float2(q22[j], q22[j + H]);
-    }
-    const float2 th2 = make_float2(tp.theta, tp.theta);
-    float2 t12[H], t22[H], qx12[H], qx22[H], qy12[H], qy22[H];
-    const int fnext = min(ty * R + R, FH - 1);     // the thread below's first row
-    const int fprev = max(ty * R - 1, 0);          // the thread above's last row
-#pragma unroll 1
-    for (int it = 0; it < n_iters; ++it) {
-#pragma unroll
-      for (int j = 0; j < H; ++j) {
-        const int f0 = ty * R + j, f1 = f0 + H;
-        const bool last = j + 1 == H;
-        const float2 ub_b = last ? make_float2(ub2[0].y, s_ub[fnext][tx]) : ub2[j + 1];
-        const float2 vb1_b = last ? make_float2(vb12[0].y, s_vb1[fnext][tx]) : vb12[j + 1];
-        const float2 vb2_b = last ? make_float2(vb22[0].y, s_vb2[fnext][tx]) : vb22[j + 1];
-        tgv_px_dual2<FTZ>(mb >> (3 * j), mb >> (3 * (j + H)), ub2[j],
-                     make_float2(s_ub[f0][txr], s_ub[f1][txr]), ub_b, vb12[j],
-                     make_float2(s_vb1[f0][txr], s_vb1[f1][txr]), vb1_b, vb22[j],
-                     make_float2(s_vb2[f0][txr], s_vb2[f1][txr]), vb2_b, c2[j], tp, p12[j],
-                     p22[j], q112[j], q122[j], q212[j], q222[j], t12[j], t22[j], qx12[j],
-                     qx22[j], qy12[j], qy22[j]);
-        s_t1[f0][tx] = t12[j].x;   s_t1[f1][tx] = t12[j].y;
-        s_t2[f0][tx] = t22[j].x;   s_t2[f1][tx] = t22[j].y;
-        s_qx1[f0][tx] = qx12[j].x; s_qx1[f1][tx] = qx12[j].y;
-        s_qx2[f0][tx] = qx22[j].x; s_qx2[f1][tx] = qx22[j].y;
-        s_qy1[f0][tx] = qy12[j].x; s_qy1[f1][tx] = qy12[j].y;
-        s_qy2[f0][tx] = qy22[j].x; s_qy2[f1][tx] = qy22[j].y;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < H; ++j) {
-        const int f0 = ty * R + j, f1 = f0 + H;
-        // above: the previous pair, or for the first pair the thread above's
-        // last row (the footprint's top row reads itself) and row H - 1
-        const float2 t2_u = j > 0 ? t22[j - 1] : make_float2(s_t2[fprev][tx], t22[H - 1].x);
-        const float2 qy1_u = j > 0 ? qy12[j - 1] : make_float2(s_qy1[fprev][tx], qy12[H - 1].x);
-        const float2 qy2_u = j > 0 ? qy22[j - 1] : make_float2(s_qy2[fprev][tx], qy22[H - 1].x);
-        tgv_px_primal2(t12[j], make_float2(s_t1[f0][txl], s_t1[f1][txl]), t22[j], t2_u,
-                       qx12[j], make_float2(s_qx1[f0][txl], s_qx1[f1][txl]), qy12[j], qy1_u,
-                       qx22[j], make_float2(s_qx2[f0][txl], s_qx2[f1][txl]), qy22[j], qy2_u,
-                       p12[j], p22[j], c2[j], th2, u2[j], ub2[j], v12[j], v22[j], vb12[j],
-                       vb22[j]);
-        s_ub[f0][tx] = ub2[j].x;   s_ub[f1][tx] = ub2[j].y;
-        s_vb1[f0][tx] = vb12[j].x; s_vb1[f1][tx] = vb12[j].y;
-        s_vb2[f0][tx] = vb22[j].x; s_vb2[f1][tx] = vb22[j].y;
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-      u[j] = u2[j].x;     u[j + H] = u2[j].y;
-      ub[j] = ub2[j].x;   ub[j + H] = ub2[j].y;
-      v1[j] = v12[j].x;   v1[j + H] = v12[j].y;
-      v2[j] = v22[j].x;   v2[j + H] = v22[j].y;
-      vb1[j] = vb12[j].x; vb1[j + H] = vb12[j].y;
-      vb2[j] = vb22[j].x; vb2[j + H] = vb22[j].y;
-      p1[j] = p12[j].x;   p1[j + H] = p12[j].y;
-      p2[j] = p22[j].x;   p2[j + H] = p22[j].y;
-      q11[j] = q112[j].x; q11[j + H] = q112[j].y;
-      q12[j] = q122[j].x; q12[j + H] = q122[j].y;
-      q21[j] = q212[j].x; q21[j + H] = q212[j].y;
-      q22[j] = q222[j].x; q22[j + H] = q222[j].y;
-    }
-  } else {
-  float t1[R], t2[R], qx1[R], qx2[R], qy1[R], qy2[R];
-#pragma unroll 1
-  for (int it = 0; it < n_iters; ++it) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int fy = ty * R + r;
-      const int fb = min(fy + 1, FH - 1);
-      const float ub_b = (r + 1 < R) ? ub[r + 1] : s_ub[fb][tx];
-      const float vb1_b = (r + 1 < R) ? vb1[r + 1] : s_vb1[fb][tx];
-      const float vb2_b = (r + 1 < R) ? vb2[r + 1] : s_vb2[fb][tx];
-      tgv_px_dual<FTZ>(mb >> (3 * r), ub[r], s_ub[fy][txr], ub_b, vb1[r], s_vb1[fy][txr], vb1_b,
-                  vb2[r], s_vb2[fy][txr], vb2_b, c[r], tp, p1[r], p2[r], q11[r], q12[r],
-                  q21[r], q22[r], t1[r], t2[r], qx1[r], qx2[r], qy1[r], qy2[r]);
-      s_t1[fy][tx] = t1[r];
-      s_t2[fy][tx] = t2[r];
-      s_qx1[fy][tx] = qx1[r];
-      s_qx2[fy][tx] = qx2[r];
-      s_qy1[fy][tx] = qy1[r];
-      s_qy2[fy][tx] = qy2[r];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int fy = ty * R + r;
-      const int fu = max(fy - 1, 0);
-      const float t2_u = r > 0 ? t2[r - 1] : s_t2[fu][tx];
-      const float qy1_u = r > 0 ? qy1[r - 1] : s_qy1[fu][tx];
-      const float qy2_u = r > 0 ? qy2[r - 1] : s_qy2[fu][tx];
-      tgv_px_primal(t1[r], s_t1[fy][txl], t2[r], t2_u, qx1[r], s_qx1[fy][txl], qy1[r], qy1_u,
-                    qx2[r], s_qx2[fy][txl], qy2[r], qy2_u, p1[r], p2[r], c[r], tp.theta,
-                    u[r], ub[r], v1[r], v2[r], vb1[r], vb2[r]);
-      s_ub[fy][tx] = ub[r];
-      s_vb1[fy][tx] = vb1[r];
-      s_vb2[fy][tx] = vb2[r];
-    }
-    __syncthreads();
-  }
-  }
+  // every pixel of the footprint in the FOV with both forward neighbours: the
+  // loop without the mask selects gives the same bits
+  const bool full = mb == (R == 1 ? 7u : R == 2 ? 077u : 07777u);
+  if (__syncthreads_and(full))
+    tgv_iterate<FW, NY, R, FTZ, false>(tp, n_iters, tx, ty, mb, c, s, sm);
+  else
+    tgv_iterate<FW, NY, R, FTZ, true>(tp, n_iters, tx, ty, mb, c, s, sm);
 
   if (!col_in || tx < B || tx >= FW - B) return;
 #pragma unroll
@@ -342,8 +419,8 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
     const int fy = ty * R + r;
     if (fy < B || fy >= FH - B || !ok[r]) continue;
     const unsigned k = idx[r];
-    const float a[12] = {u[r], ub[r], v1[r], v2[r], vb1[r], vb2[r], p1[r], p2[r],
-                         q11[r], q12[r], q21[r], q22[r]};
+    const float a[12] = {s.u[r],  s.ub[r], s.v1[r],  s.v2[r],  s.vb1[r], s.vb2[r],
+                         s.p1[r], s.p2[r], s.q11[r], s.q12[r], s.q21[r], s.q22[r]};
 #pragma unroll
     for (int j = 0; j < 12; ++j) out.s[j][k] = a[j];
   }
@@ -384,12 +461,13 @@ TgvState alternate(const LevelView& L) {
   return s;
 }
 
-template <int FW, int NY, int R, bool FTZ>
+template <int FW, int NY, int R, int MB, bool FTZ, bool IDLE>
 cudaError_t launch_blocked_f(const LevelView& L, const TgvState& in, const TgvState& out,
-                             const TgvParams& tp, int B, int n, bool chained, cudaStream_t st) {
+                             const TgvParams& tp, int B, int n, bool chained, int idle,
+                             cudaStream_t st) {
   const int IW = FW - 2 * B, IH = NY * R - 2 * B;
   if (IW <= 0 || IH <= 0 || n < 0 || n > B) return cudaErrorInvalidValue;
-  constexpr size_t smem = 9 * (size_t)FW * NY * R * sizeof(float);
+  constexpr size_t smem = sizeof(TgvShared<FW, NY, R>);
   if constexpr (smem > 48 * 1024) {      // above the default limit: opt in once per device
     static std::atomic<unsigned long long> opted{0};
     int dev = 0;
@@ -397,7 +475,7 @@ cudaError_t launch_blocked_f(const LevelView& L, const TgvState& in, const TgvSt
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(opted.load() & bit)) {
-      e = cudaFuncSetAttribute(k_tgv_blocked<FW, NY, R, FTZ>,
+      e = cudaFuncSetAttribute(k_tgv_blocked<FW, NY, R, MB, FTZ, IDLE>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
       opted.fetch_or(bit);
@@ -413,42 +491,68 @@ cudaError_t launch_blocked_f(const LevelView& L, const TgvState& in, const TgvSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_tgv_blocked<FW, NY, R, FTZ>, L, in, out, tp, B, n,
-                            chained ? 1 : 0);
+  return cudaLaunchKernelEx(&cfg, k_tgv_blocked<FW, NY, R, MB, FTZ, IDLE>, L, in, out, tp, B, n,
+                            chained ? 1 : 0, idle);
 }
 
-template <int FW, int NY, int R>
+// SKIP: also instantiated without the footprints outside the FOV.
+template <int FW, int NY, int R, int MB = (FW * NY >= 512 ? 1 : 2), bool SKIP = false>
 cudaError_t launch_blocked_t(const LevelView& L, const TgvState& in, const TgvState& out,
-                             const TgvParams& tp, int B, int n, bool chained, cudaStream_t st) {
-  return tgv_normal_radii(tp)
-             ? launch_blocked_f<FW, NY, R, true>(L, in, out, tp, B, n, chained, st)
-             : launch_blocked_f<FW, NY, R, false>(L, in, out, tp, B, n, chained, st);
+                             const TgvParams& tp, int B, int n, bool chained, int idle,
+                             cudaStream_t st) {
+  const bool ftz = tgv_normal_radii(tp);
+  if constexpr (SKIP) {
+    if (idle >= 0)
+      return ftz ? launch_blocked_f<FW, NY, R, MB, true, true>(L, in, out, tp, B, n, chained, idle, st)
+                 : launch_blocked_f<FW, NY, R, MB, false, true>(L, in, out, tp, B, n, chained, idle, st);
+  }
+  return ftz ? launch_blocked_f<FW, NY, R, MB, true, false>(L, in, out, tp, B, n, chained, idle, st)
+             : launch_blocked_f<FW, NY, R, MB, false, false>(L, in, out, tp, B, n, chained, idle, st);
 }
 
 // The 32 x 32 footprint on 256 threads of 4 rows (variant 0), 1024 threads
 // of 1 row (1) or 512 threads of 2 rows (2): more threads shorten each
 // thread's dependent chain per iteration on the latency-bound levels.  The
 // 64 x 32 footprint on 512 threads of 4 rows (3) or 1024 threads of 2 rows
-// (4): less halo recomputed per interior pixel on the large levels (72 KB
-// of shared memory).
+// (4): less halo recomputed per interior pixel on the large levels.  Only
+// the automatic schedule uses 32 x 16 on 512 threads (5), 32 x 24 on 768 (6)
+// and 32 x 48 on 768 of 2 rows (7).
 cudaError_t launch_blocked(int variant, const LevelView& L, const TgvState& in,
                            const TgvState& out, const TgvParams& tp, int B, int n, bool chained,
-                           cudaStream_t st) {
+                           int idle, cudaStream_t st) {
+#define FS_TGV(...) return launch_blocked_t<__VA_ARGS__>(L, in, out, tp, B, n, chained, idle, st)
   switch (variant) {
-    case 0: return launch_blocked_t<32, 8, 4>(L, in, out, tp, B, n, chained, st);
-    case 1: return launch_blocked_t<32, 32, 1>(L, in, out, tp, B, n, chained, st);
-    case 2: return launch_blocked_t<32, 16, 2>(L, in, out, tp, B, n, chained, st);
-    case 3: return launch_blocked_t<64, 8, 4>(L, in, out, tp, B, n, chained, st);
-    case 4: return launch_blocked_t<64, 16, 2>(L, in, out, tp, B, n, chained, st);
+    case 0: FS_TGV(32, 8, 4, 2, true);
+    case 1: FS_TGV(32, 32, 1);
+    case 2: FS_TGV(32, 16, 2);
+    case 3: FS_TGV(64, 8, 4, 1, true);
+    case 4: FS_TGV(64, 16, 2);
+    case 5: FS_TGV(32, 16, 1);
+    case 6: FS_TGV(32, 24, 1);
+    case 7: FS_TGV(32, 24, 2, 1, true);
     default: return cudaErrorInvalidValue;
   }
+#undef FS_TGV
 }
 
 }  // namespace
 
-cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, int B, int variant,
+// Fitted as pd_auto's table.  What it picks against the fixed choice it
+// replaces (32 x 32 footprints of 256 threads at depth 4), us per 10 / 100
+// iterations: 50 x 50 9.5 / 58.6 against 18.2 / 118.7, 200 x 200 11.2 / 89.9
+// against 18.7 / 138.5, 512 x 512 35.6 / 309 against 45.4 / 339.
+PdSchedule tgv_auto(const LevelView& L, int iters, int launches, int sms) {
+  static const BlockFit kFit[] = {
+      {5, 32, 16, 1, 2.3f, 0.24f, false}, {6, 32, 24, 1, 2.7f, 0.36f, false},
+      {2, 32, 32, 1, 3.0f, 0.46f, false}, {7, 32, 48, 1, 3.3f, 0.70f, true},
+      {3, 64, 32, 1, 5.3f, 0.78f, true},  {0, 32, 32, 2, 3.3f, 0.95f, true},
+  };
+  return block_schedule(kFit, (int)(sizeof(kFit) / sizeof(kFit[0])), L, iters, launches, sms);
+}
+
+cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, const PdSchedule& ps,
                                   int n, cudaStream_t st) {
-  if (B <= 0) {                       // a dual and a primal launch per iteration
+  if (ps.launches <= 0) {             // a dual and a primal launch per iteration
     const dim3 g = tgrid(L.W, L.H), b(32, 8);
     for (int k = 0; k < n; ++k) {
       k_tgv_dual<<<g, b, 0, st>>>(L, tp);
@@ -456,16 +560,15 @@ cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, int B
     }
     return cudaGetLastError();
   }
-  // temporal blocking: at most B iterations per launch, an even number of
-  // launches (when n >= 2) so that the state ends in the level's planes
-  int nl = (n + B - 1) / B;
-  if (nl % 2 == 1 && n >= 2) ++nl;
+  // temporal blocking: an even number of launches (when n >= 2), so that the
+  // state ends in the level's planes
+  const int nl = ps.launches;
   const TgvState A = primary(L), Bs = alternate(L);
   for (int k = 0, done = 0; k < nl; ++k) {
     int m = (n - done) / (nl - k);
     if ((n - done) % (nl - k)) ++m;
-    cudaError_t e = launch_blocked(variant, L, (k % 2 == 0) ? A : Bs, (k % 2 == 0) ? Bs : A,
-                                   tp, B, m, k > 0, st);
+    cudaError_t e = launch_blocked(ps.variant, L, (k % 2 == 0) ? A : Bs, (k % 2 == 0) ? Bs : A,
+                                   tp, ps.depth, m, k > 0, !ps.skip ? -1 : k == 0 ? n : 0, st);
     if (e != cudaSuccess) return e;
     done += m;
   }

@@ -79,7 +79,9 @@ __device__ __forceinline__ float tgv_ball(float n2, float r) {
 
 // Dual ascent at one pixel from its own and its right (r) / lower (b)
 // neighbours' ubar, vbar.  Updates p, q; returns t and the masked q.
-template <bool FTZ>
+// MASKED = false: a pixel whose mask bits are all set (the selects would give
+// every value as it is).
+template <bool FTZ, bool MASKED = true>
 __device__ __forceinline__ void tgv_px_dual(unsigned m, float ub, float ub_r, float ub_b,
                                             float vb1, float vb1_r, float vb1_b, float vb2,
                                             float vb2_r, float vb2_b, const TgvConst& c,
@@ -87,7 +89,7 @@ __device__ __forceinline__ void tgv_px_dual(unsigned m, float ub, float ub_r, fl
                                             float& q11, float& q12, float& q21, float& q22,
                                             float& t1, float& t2, float& qx1, float& qx2,
                                             float& qy1, float& qy2) {
-  const bool gx = m & MASK_GX, gy = m & MASK_GY;
+  const bool gx = !MASKED || (m & MASK_GX), gy = !MASKED || (m & MASK_GY);
   const float g1 = gx ? __fsub_rn(ub_r, ub) : 0.f;
   const float g2 = gy ? __fsub_rn(ub_b, ub) : 0.f;
   const float d = fmaf(c.sx, g1, __fmul_rn(c.sy, g2));
@@ -176,13 +178,14 @@ __device__ __forceinline__ float2 tgv_sel2(bool kx, bool ky, float2 v) {
 }
 
 // m0, m1: the two pixels' mask bits.
-template <bool FTZ>
+template <bool FTZ, bool MASKED = true>
 __device__ __forceinline__ void tgv_px_dual2(
     unsigned m0, unsigned m1, float2 ub, float2 ub_r, float2 ub_b, float2 vb1, float2 vb1_r,
     float2 vb1_b, float2 vb2, float2 vb2_r, float2 vb2_b, const TgvConst2& c,
     const TgvParams& tp, float2& p1, float2& p2, float2& q11, float2& q12, float2& q21,
     float2& q22, float2& t1, float2& t2, float2& qx1, float2& qx2, float2& qy1, float2& qy2) {
-  const bool gx0 = m0 & MASK_GX, gx1 = m1 & MASK_GX, gy0 = m0 & MASK_GY, gy1 = m1 & MASK_GY;
+  const bool gx0 = !MASKED || (m0 & MASK_GX), gx1 = !MASKED || (m1 & MASK_GX);
+  const bool gy0 = !MASKED || (m0 & MASK_GY), gy1 = !MASKED || (m1 & MASK_GY);
   const float2 g1 = tgv_sel2(gx0, gx1, tgv_sub2(ub_r, ub));
   const float2 g2 = tgv_sel2(gy0, gy1, tgv_sub2(ub_b, ub));
   const float2 d = __ffma2_rn(c.sx, g1, __fmul2_rn(c.sy, g2));

@@ -15,11 +15,11 @@ from gpu_helpers import f32pair, make_solver, np64
 pytestmark = pytest.mark.gpu
 
 
-def _run(pair, choice, iters, **prm):
+def _run(pair, choice, iters, bufs=("U", "UBAR", "P"), **prm):
     s = make_solver(pair, levels=1, **prm)
     s.set_schedule([choice])
     s.solve(pair["I0"], pair["I1"], 4, iters)
-    out = [np64(s.read(0, b)) for b in ("U", "UBAR", "P")]
+    out = [np64(s.read(0, b)) for b in bufs]
     s.close()
     return out
 
@@ -69,6 +69,47 @@ def test_footprints_outside_the_fov(W, H, iters, prm):
         outs.append([np64(s.read(0, b)) for b in state])
         s.solve(p["I0"], p["I1"], 2, iters)
         outs[-1] += [np64(s.read(0, b)) for b in state]
+        s.close()
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
+TGV = ("U", "UBAR", "V", "VBAR", "P", "Q")
+
+
+@pytest.mark.parametrize("W, H, iters", [
+    (33, 21, 1), (33, 21, 2), (50, 50, 100), (100, 90, 30), (200, 200, 100), (256, 256, 10),
+    (401, 333, 30), (512, 512, 30), (900, 700, 11)])
+def test_automatic_tgv_schedule_equals_a_launch_per_step(W, H, iters):
+    p = f32pair(synth.plain_small(1, W=W, H=H, supersample=1))
+    for a, b in zip(_run(p, -1, iters, TGV, regularizer="tgv"),
+                    _run(p, 0, iters, TGV, regularizer="tgv")):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prm", [dict(), dict(precond=0, theta=0.5)])
+@pytest.mark.parametrize("W, H, iters", [(1100, 900, 12), (700, 1100, 31)])
+def test_tgv_footprints_outside_the_fov(W, H, iters, prm):
+    # as above: state at rest and not at rest outside a small FOV circle
+    cam = dict(model="equidistant", fx=120.0, fy=130.0, cx=400.3, cy=520.8, k=[0] * 4, fov_deg=170.0)
+    rng = np.random.default_rng(6)
+    p = dict(I0=rng.random((H, W)), I1=rng.random((H, W)), cam0=cam, cam1=dict(cam), R=np.eye(3),
+             t=np.array([-0.1, 0.0, 0.0]), levels=1)
+    shape = dict(U=(H, W), UBAR=(H, W), V=(2, H, W), VBAR=(2, H, W), P=(2, H, W), Q=(4, H, W))
+    state = {b: rng.uniform(-1.5, 1.5, shape[b]) for b in TGV}
+    outs = []
+    for choice in (-1, 0):
+        s = make_solver(p, levels=1, regularizer="tgv", **prm)
+        s.set_schedule([choice])
+        s.solve(p["I0"], p["I1"], 1, 2)
+        M = np64(s.read(0, "MASK")) > 0.5
+        for b, v in state.items():
+            s.write(0, b, v)
+        s.stage(0, "PD", iters)
+        # (a launch per step leaves the pixels outside the FOV as they are)
+        outs.append([np64(s.read(0, b))[..., M] for b in TGV])
+        s.solve(p["I0"], p["I1"], 2, iters)
+        outs[-1] += [np64(s.read(0, b)) for b in TGV]
         s.close()
     for a, b in zip(*outs):
         assert np.array_equal(a, b)
