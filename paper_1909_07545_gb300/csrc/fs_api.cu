@@ -543,6 +543,10 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
   }
   if (h->prm.regularizer == FS_REG_TGV) {
     TgvParams tp{h->prm.lambda, h->prm.theta, h->prm.alpha0, h->prm.alpha1, h->prm.precond};
+    if (L.consts_stale) {
+      FS_LAUNCH("k_tgv_consts", launch_tgv_consts(L.v, tp.lam, tp.precond, st));
+      L.consts_stale = false;
+    }
     FS_LAUNCH("k_tgv", launch_tgv_iterations(L.v, tp, pd_plan(h, l, iters), iters, st));
     return FS_OK;
   }
@@ -596,7 +600,9 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
 fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
                     bool chain = false) {
   HostLevel& L = h->lv[l];
-  const int consts = h->prm.regularizer == FS_REG_TGV ? 0 : 1;
+  const int consts = h->prm.regularizer != FS_REG_TGV ? WARP_CONSTS_HUBER
+                     : h->prm.precond                 ? WARP_CONSTS_TGV
+                                                      : WARP_CONSTS_TGV_SCALAR;
   // every stage but the iterations and the warp starts can change sigma,
   // tau, I_u, rho0 or u_w
   if (stage != FS_STAGE_PD && stage != FS_STAGE_WARP && stage != FS_STAGE_CLIP_WARP)
@@ -617,9 +623,7 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
     case FS_STAGE_WARP:
       FS_LAUNCH("k_warp", launch_warp(L.v, h->prm.deriv == FS_DERIV_CENTRAL, h->prm.lambda,
                                       h->prm.huber_eps, consts, st));
-      L.consts_stale = !consts;
-      if (h->prm.regularizer == FS_REG_TGV)
-        FS_LAUNCH("k_tgv_warp_start", launch_tgv_warp_start(L.v, st));
+      L.consts_stale = false;
       return FS_OK;
     case FS_STAGE_PD: {
       if (count < 1) return fail(FS_EINVAL, "pd: count must be >= 1");
@@ -633,9 +637,7 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
       FS_LAUNCH("k_clip_warp", launch_clip_warp(L.v, h->prm.du_max,
                                                 h->prm.deriv == FS_DERIV_CENTRAL, h->prm.lambda,
                                                 h->prm.huber_eps, consts, chain, st));
-      L.consts_stale = !consts;
-      if (h->prm.regularizer == FS_REG_TGV)
-        FS_LAUNCH("k_tgv_warp_start", launch_tgv_warp_start(L.v, st));
+      L.consts_stale = false;
       return FS_OK;
     case FS_STAGE_WARM:
       FS_LAUNCH("k_warm_start", launch_warm_start(L.v, h->prm.du_max, st));

@@ -102,22 +102,25 @@ int pd_launch_count(int iters, int depth);
 // primal launch each, else temporally blocked on the footprint ps.variant --
 // 0..4, the encoding of fs_autotune: 32 x 32 of 256 (variant 0), 1024 (1) or
 // 512 (2) threads, 64 x 32 of 512 (3) or 1024 (4) threads; further ones of
-// tgv_auto (identical results); v, vbar, q <- 0; vbar <- v at a warp's start.
+// tgv_auto (identical results).  The blocked kernel reads
+// the constants launch_tgv_consts or the warp start wrote.  v, vbar, q <- 0.
 constexpr int kTgvVariants = 5;
 struct TgvParams;
 cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, const PdSchedule& ps,
                                   int n, cudaStream_t st);
 cudaError_t launch_tgv_reset(const LevelView& L, cudaStream_t st);
+cudaError_t launch_tgv_consts(const LevelView& L, float lam, int precond, cudaStream_t st);
 // Energy terms of a level summed into acc[0..2] (data, regulariser, L1
 // residual); acc must be zeroed first (k_energy.cu).
 cudaError_t launch_energy(const LevelView& L, float lam, float eps, int tgv, float alpha0,
                           float alpha1, double* acc, cudaStream_t st);
-cudaError_t launch_tgv_warp_start(const LevelView& L, cudaStream_t st);
 cudaError_t launch_tensor(const LevelView& L, float beta, float eta, int precond,
                           cudaStream_t st);
-// consts = 1: also the per-warp constants of the primal-dual iterations
-// (the values launch_pd_consts computes), from the I_u, rho0 and u_w the
-// kernel writes.
+// consts (WarpConsts): also the per-warp constants of the primal-dual
+// iterations, from the I_u, rho0 and u_w the kernel writes: Huber-TV's (the
+// values launch_pd_consts computes), or TGV's with preconditioned or scalar
+// steps (launch_tgv_consts) and vbar <- v.
+enum WarpConsts { WARP_CONSTS_HUBER = 1, WARP_CONSTS_TGV = 2, WARP_CONSTS_TGV_SCALAR = 3 };
 cudaError_t launch_warp(const LevelView& L, int central, float lam, float eps, int consts,
                         cudaStream_t st);
 // k_clip of one warp fused with k_warp of the next (same results).  chained:

@@ -5,6 +5,7 @@
 #include "fs_kernels.h"
 #include "level_px.cuh"
 #include "pd_math.cuh"
+#include "pd_tgv_math.cuh"
 
 namespace fs {
 
@@ -273,9 +274,45 @@ __device__ __forceinline__ void pd_consts_px(const LevelView& L, size_t i, float
   L.c0[i] = c.c0;
 }
 
-// consts: also write the per-warp constants of the primal-dual iterations
-// (pd_consts_px; Huber-TV handles).
-template <int S>
+// The same for the TGV iterations (tgv_const of the stored values): sigma_p in
+// L.dinv, tau_v in L.sd, the L1 step and c0 in their planes; and vbar <- v.
+__device__ __forceinline__ void tgv_consts_px(const LevelView& L, int x, int y, size_t i,
+                                              float Iu, float rho0, float uw, float lam,
+                                              int precond) {
+  const unsigned ml = x > 0 ? L.mask[i - 1] : 0u, mu = y > 0 ? L.mask[i - L.P] : 0u;
+  const TgvParams tp{lam, 0.f, 0.f, 0.f, precond};
+  TgvConst c;
+  tgv_const(L.mask[i], ml, mu, 0.f, 0.f, L.sig[i], L.tau[i], Iu, rho0, uw, tp, c);
+  L.dinv[i] = c.sp;
+  L.sd[i] = c.tv;
+  L.step[i] = c.step;
+  L.c0[i] = c.c0;
+}
+
+// What a warp start writes for the iterations (enum WarpConsts; TGV: one of
+// its two).
+template <int S, bool CG, bool TGV>
+__device__ __forceinline__ void warp_consts_px(const LevelView& L, int x, int y, size_t i,
+                                               float Iu, float rho0, float u, float lam,
+                                               float eps, int consts) {
+  if constexpr (!TGV) {
+    pd_consts_px<S, CG>(L, i, Iu, rho0, u, lam, eps);
+  } else {
+    tgv_consts_px(L, x, y, i, Iu, rho0, u, lam, consts == WARP_CONSTS_TGV);
+    L.vb1[i] = L.v1[i];
+    L.vb2[i] = L.v2[i];
+  }
+}
+
+__global__ void k_tgv_consts(LevelView L, float lam, int precond) {
+  int x = blockIdx.x * blockDim.x + threadIdx.x;
+  int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= L.W || y >= L.H) return;
+  size_t i = (size_t)y * L.P + x;
+  tgv_consts_px(L, x, y, i, sld<ST_F32>(L.Iu, i), sld<ST_F32>(L.rho0, i), L.uw[i], lam, precond);
+}
+
+template <int S, bool TGV>
 __global__ void k_warp(LevelView L, int central, float lam, float eps, int consts) {
   int x = blockIdx.x * blockDim.x + threadIdx.x;
   int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -290,7 +327,7 @@ __global__ void k_warp(LevelView L, int central, float lam, float eps, int const
   float u = L.u[i];
   L.ubar[i] = u;
   L.uw[i] = u;
-  if (consts) pd_consts_px<S>(L, i, Iu, rho0, u, lam, eps);
+  warp_consts_px<S, false, TGV>(L, x, y, i, Iu, rho0, u, lam, eps, consts);
 }
 
 // ------------------------------------------------------------ clip + update
@@ -322,7 +359,7 @@ __global__ void k_clip(LevelView L, float du_max) {
 // k_warp at every pixel, with the updated w and u kept in registers (each
 // pixel's clip and linearisation read only that pixel's state; the gathers
 // read I1 and gamma', which neither writes).
-template <int S, bool CHAIN>
+template <int S, bool CHAIN, bool TGV>
 __global__ void k_clip_warp(LevelView L, float du_max, int central, float lam, float eps,
                             int consts) {
   if constexpr (CHAIN) {
@@ -350,7 +387,7 @@ __global__ void k_clip_warp(LevelView L, float du_max, int central, float lam, f
   L.g[i] = g;
   L.ubar[i] = u;
   L.uw[i] = u;
-  if (consts) pd_consts_px<S, CHAIN>(L, i, Iu, rho0, u, lam, eps);
+  warp_consts_px<S, CHAIN, TGV>(L, x, y, i, Iu, rho0, u, lam, eps, consts);
 }
 
 
@@ -507,17 +544,28 @@ cudaError_t launch_tensor(const LevelView& L, float beta, float eta, int precond
 }
 cudaError_t launch_warp(const LevelView& L, int central, float lam, float eps, int consts,
                         cudaStream_t st) {
-  FS_STORAGE_SWITCH(L.st, (k_warp<S><<<grid_of(L.W, L.H), kBlk, 0, st>>>(L, central, lam, eps,
-                                                                        consts)))
+  if (consts != WARP_CONSTS_HUBER) {            // TGV: FP32 storage only
+    k_warp<ST_F32, true><<<grid_of(L.W, L.H), kBlk, 0, st>>>(L, central, lam, eps, consts);
+    return cudaGetLastError();
+  }
+  FS_STORAGE_SWITCH(L.st, (k_warp<S, false><<<grid_of(L.W, L.H), kBlk, 0, st>>>(
+                              L, central, lam, eps, consts)))
+}
+
+cudaError_t launch_tgv_consts(const LevelView& L, float lam, int precond, cudaStream_t st) {
+  k_tgv_consts<<<grid_of(L.W, L.H), kBlk, 0, st>>>(L, lam, precond);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_clip_warp(const LevelView& L, float du_max, int central, float lam, float eps,
                              int consts, bool chained, cudaStream_t st) {
-  FS_STORAGE_SWITCH(L.st,
-                    return chained ? launch_chained(k_clip_warp<S, true>, L, true, st, L, du_max,
-                                                    central, lam, eps, consts)
-                                   : launch_chained(k_clip_warp<S, false>, L, false, st, L, du_max,
-                                                    central, lam, eps, consts))
+  if (consts != WARP_CONSTS_HUBER)
+    return launch_chained(k_clip_warp<ST_F32, false, true>, L, false, st, L, du_max, central, lam,
+                          eps, consts);
+  FS_STORAGE_SWITCH(L.st, return launch_chained(chained ? k_clip_warp<S, true, false>
+                                                        : k_clip_warp<S, false, false>,
+                                                L, chained, st, L, du_max, central, lam, eps,
+                                                consts))
 }
 cudaError_t launch_clip(const LevelView& L, float du_max, bool chained, cudaStream_t st) {
   return chained ? launch_chained(k_clip<true>, L, true, st, L, du_max)

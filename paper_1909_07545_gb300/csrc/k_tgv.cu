@@ -352,36 +352,36 @@ k_tgv_blocked(LevelView L, TgvState in, TgvState out, TgvParams tp, int B, int n
   TgvConst c[R];
   unsigned mb = 0;
   {
-    // every load first, from clamped addresses (the left / upper neighbour
-    // of column / row 0 is read as the pixel itself and its bits dropped),
-    // then the constants: a thread's loads are all in flight together
-    float sx[R], sy[R], sg[R], ta[R], iu[R], r0[R], uw[R];
-    unsigned m[R], ml[R], mu[R];
-    const unsigned dl = gxc > 0 ? 1u : 0u;
+    // every load first, from clamped addresses, then the selection: a
+    // thread's loads are all in flight together
+    float sx[R], sy[R], sp[R], ta[R], st[R], c0[R], tv[R];
+    unsigned m[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int gy = oy + ty * R + r;
       ok[r] = col_in && gy >= 0 && gy < L.H;
-      const int gyc = min(max(gy, 0), L.H - 1);
-      idx[r] = (unsigned)(gyc * L.P + gxc);
-      const unsigned du = gyc > 0 ? (unsigned)L.P : 0u;
+      idx[r] = (unsigned)(min(max(gy, 0), L.H - 1) * L.P + gxc);
       sx[r] = sld<ST_F32>(L.sx, idx[r]);
       sy[r] = sld<ST_F32>(L.sy, idx[r]);
-      sg[r] = L.sig[idx[r]];
+      sp[r] = L.dinv[idx[r]];
       ta[r] = L.tau[idx[r]];
-      iu[r] = sld<ST_F32>(L.Iu, idx[r]);
-      r0[r] = sld<ST_F32>(L.rho0, idx[r]);
-      uw[r] = L.uw[idx[r]];
+      st[r] = L.step[idx[r]];
+      c0[r] = L.c0[idx[r]];
+      tv[r] = L.sd[idx[r]];
       m[r] = L.mask[idx[r]];
-      ml[r] = L.mask[idx[r] - dl];
-      mu[r] = L.mask[idx[r] - du];
-      if (!dl) ml[r] = 0u;
-      if (!du) mu[r] = 0u;
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const unsigned mm = ok[r] ? m[r] : 0u;
-      tgv_const(mm, ml[r], mu[r], sx[r], sy[r], sg[r], ta[r], iu[r], r0[r], uw[r], tp, c[r]);
+      const bool in_fov = mm & MASK_IN;          // off the FOV nothing moves
+      c[r].sx = in_fov ? sx[r] : 0.f;
+      c[r].sy = in_fov ? sy[r] : 0.f;
+      c[r].sp = in_fov ? sp[r] : 0.f;
+      c[r].sq = in_fov ? (tp.precond ? 0.5f : kTgvScalarStep) : 0.f;
+      c[r].tau = in_fov ? (tp.precond ? ta[r] : kTgvScalarStep) : 0.f;
+      c[r].step = in_fov ? st[r] : 0.f;
+      c[r].c0 = in_fov ? c0[r] : 0.f;
+      c[r].tv = in_fov ? tv[r] : 0.f;
       mb |= mm << (3 * r);
     }
   }
@@ -434,16 +434,6 @@ __global__ void k_tgv_reset(LevelView L) {
   const size_t i = (size_t)y * L.P + x;
   L.v1[i] = L.v2[i] = L.vb1[i] = L.vb2[i] = 0.f;
   L.q11[i] = L.q12[i] = L.q21[i] = L.q22[i] = 0.f;
-}
-
-// vbar <- v at the start of a warp (as ubar <- u).
-__global__ void k_tgv_warp_start(LevelView L) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  if (x >= L.W || y >= L.H) return;
-  const size_t i = (size_t)y * L.P + x;
-  L.vb1[i] = L.v1[i];
-  L.vb2[i] = L.v2[i];
 }
 
 namespace {
@@ -584,11 +574,6 @@ cudaError_t launch_tgv_iterations(const LevelView& L, const TgvParams& tp, const
 
 cudaError_t launch_tgv_reset(const LevelView& L, cudaStream_t st) {
   k_tgv_reset<<<tgrid(L.W, L.H), dim3(32, 8), 0, st>>>(L);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_tgv_warp_start(const LevelView& L, cudaStream_t st) {
-  k_tgv_warp_start<<<tgrid(L.W, L.H), dim3(32, 8), 0, st>>>(L);
   return cudaGetLastError();
 }
 
