@@ -350,15 +350,29 @@ fs_status upload_masks(fs_handle* h, std::vector<uint8_t>& host) {
   return FS_OK;
 }
 
-// gamma' of level l (k_trajectory) with the level's camera and the unit
-// direction of t' as float-float words.
-fs_status launch_trajectory(fs_handle* h, int l, cudaStream_t st) {
-  HostLevel& L = h->lv[l];
-  double n = std::sqrt(h->tp[0] * h->tp[0] + h->tp[1] * h->tp[1] + h->tp[2] * h->tp[2]);
-  k_trajectory<<<grid2(L.W, L.H), kBlock2, 0, st>>>(
-      dev_cam_df(h->cam[0], L.fx, L.fy, L.cx, L.cy), df_from_double(h->tp[0] / n),
-      df_from_double(h->tp[1] / n), df_from_double(h->tp[2] / n), L.v);
-  FS_LAUNCHED("k_trajectory");
+// gamma' of levels [first, first + n) with their cameras and the unit
+// direction of t' as float-float words, and with `field` the calibration
+// field (first = 0).
+fs_status launch_fields(fs_handle* h, int first, int n, bool field, cudaStream_t st) {
+  PoseFields F{};
+  const double t = std::sqrt(h->tp[0] * h->tp[0] + h->tp[1] * h->tp[1] + h->tp[2] * h->tp[2]);
+  F.tx = df_from_double(h->tp[0] / t);
+  F.ty = df_from_double(h->tp[1] / t);
+  F.tz = df_from_double(h->tp[2] / t);
+  F.n = n;
+  int blocks = 0;
+  for (int k = 0; k < n; ++k) {
+    const HostLevel& L = h->lv[first + k];
+    F.lv[k] = PoseLevel{dev_cam_df(h->cam[0], L.fx, L.fy, L.cx, L.cy), L.v.gamma, L.v.mask,
+                        L.W, L.H, L.P, blocks};
+    blocks += (L.W + 31) / 32 * ((L.H + 7) / 8);
+  }
+  if (field) {
+    for (int i = 0; i < 9; ++i) F.R.r[i] = df_from_double(h->pose.R[i]);
+    F.cam1 = dev_cam_df(h->cam[1], h->cam[1].fx, h->cam[1].fy, h->cam[1].cx, h->cam[1].cy);
+    F.field = h->cfield;
+  }
+  FS_LAUNCH("k_pose_fields", launch_pose_fields(F, blocks, st));
   return FS_OK;
 }
 
@@ -378,20 +392,8 @@ fs_status build_fields(fs_handle* h) {
   for (int i = 0; i < 9 && identity; ++i) identity = R[i] == ((i % 4 == 0) ? 1.0 : 0.0);
   if (identity) {       // the same lens, no rotation: c(x) = pi_0(pi_0^-1(x)) - x = 0
     FS_CUDA(cudaMemsetAsync(h->cfield, 0, (size_t)L0.P * L0.H * sizeof(float4), h->stream));
-  } else {
-    RotDF Rd;
-    for (int i = 0; i < 9; ++i) Rd.r[i] = df_from_double(R[i]);
-    k_calib_field<<<grid2(L0.W, L0.H), kBlock2, 0, h->stream>>>(
-        dev_cam_df(h->cam[0], L0.fx, L0.fy, L0.cx, L0.cy),
-        dev_cam_df(h->cam[1], h->cam[1].fx, h->cam[1].fy, h->cam[1].cx, h->cam[1].cy), Rd,
-        L0.v.mask, h->cfield, L0.W, L0.H, L0.P);
-    FS_LAUNCHED("k_calib_field");
   }
-  for (int l = 0; l < h->L; ++l) {
-    fs_status s = launch_trajectory(h, l, h->stream);
-    if (s != FS_OK) return s;
-  }
-  return FS_OK;
+  return launch_fields(h, 0, h->L, !identity, h->stream);
 }
 
 // A schedule choice of fs_autotune / fs_set_schedule: 0 = cluster (Huber-TV)
@@ -644,7 +646,7 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
       if (h->prm.regularizer == FS_REG_TGV) FS_LAUNCH("k_tgv_reset", launch_tgv_reset(L.v, st));
       return FS_OK;
     case FS_STAGE_TRAJECTORY:
-      return launch_trajectory(h, l, st);
+      return launch_fields(h, l, 1, false, st);
     default:
       return fail(FS_EINVAL, "unknown stage %d", stage);
   }

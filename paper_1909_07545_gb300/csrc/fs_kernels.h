@@ -42,9 +42,24 @@ constexpr int PD_TILE_64x32_T1024 = PD_TILE_COUNT + 6;
 constexpr int PD_TILE_64x32_T512 = PD_TILE_COUNT + 7;
 enum PDClusterVariant { PD_CLUSTER_16 = 0, PD_CLUSTER_32 = 1 };
 
-__global__ void k_trajectory(DevCamDF cam, df tx, df ty, df tz, LevelView L);
-__global__ void k_calib_field(DevCamDF c0, DevCamDF c1, RotDF R, const uint8_t* __restrict__ mask,
-                              float4* __restrict__ field, int W, int H, int P);
+// The fields of a pose (k_pose_fields): gamma' of n levels, whose 32 x 8
+// blocks follow one another in one grid, and the calibration field of the
+// first (null: not computed).
+struct PoseLevel {
+  DevCamDF cam;
+  float2* gamma;
+  const uint8_t* mask;
+  int W, H, P, first_block;
+};
+struct PoseFields {
+  PoseLevel lv[8];
+  int n;
+  df tx, ty, tz;                 // unit t'
+  DevCamDF cam1;
+  RotDF R;
+  float4* field;
+};
+cudaError_t launch_pose_fields(const PoseFields& F, int blocks, cudaStream_t st);
 __global__ void k_copy_in(const float* __restrict__ src, float* __restrict__ dst, int W, int H,
                           int P);
 __global__ void k_depth(LevelView L, DevCam cam, float Cx, float Cy, float Cz,
