@@ -597,14 +597,19 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
   return FS_OK;
 }
 
+// Which constants a warp start writes for the handle's iterations.
+int warp_consts(const fs_handle* h) {
+  return h->prm.regularizer != FS_REG_TGV ? WARP_CONSTS_HUBER
+         : h->prm.precond                 ? WARP_CONSTS_TGV
+                                          : WARP_CONSTS_TGV_SCALAR;
+}
+
 // chain: FS_STAGE_CLIP and FS_STAGE_CLIP_WARP directly behind run_pd's
 // launches on the stream.
 fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
                     bool chain = false) {
   HostLevel& L = h->lv[l];
-  const int consts = h->prm.regularizer != FS_REG_TGV ? WARP_CONSTS_HUBER
-                     : h->prm.precond                 ? WARP_CONSTS_TGV
-                                                      : WARP_CONSTS_TGV_SCALAR;
+  const int consts = warp_consts(h);
   // every stage but the iterations and the warp starts can change sigma,
   // tau, I_u, rho0 or u_w
   if (stage != FS_STAGE_PD && stage != FS_STAGE_WARP && stage != FS_STAGE_CLIP_WARP)
@@ -652,11 +657,17 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
   }
 }
 
-// The end of a warp (clip + update, Eq. 8-9) and, when another warp
-// follows, its start (warp + linearise) in one fused launch.
-fs_status clip_then_warp(fs_handle* h, int l, int iters, bool next, cudaStream_t st) {
-  return run_stage(h, l, next ? FS_STAGE_CLIP_WARP : FS_STAGE_CLIP, 0, st,
-                   short_chain(h, l, iters));
+// The start of level l: tensor and steps, the start state, the first warp's
+// linearisation.
+fs_status start_level(fs_handle* h, int l, int mode, cudaStream_t st) {
+  HostLevel& L = h->lv[l];
+  const LevelView& C = h->lv[mode == START_UPSAMPLE ? l + 1 : l].v;
+  FS_LAUNCH("k_level_start",
+            launch_level_start(mode, C, L.v, h->prm.beta, h->prm.eta, h->prm.precond,
+                               h->prm.deriv == FS_DERIV_CENTRAL, h->prm.lambda, h->prm.huber_eps,
+                               warp_consts(h), st));
+  L.consts_stale = false;
+  return FS_OK;
 }
 
 fs_status enqueue_depth(fs_handle* h, float* disp, float* depth, cudaStream_t st) {
@@ -665,6 +676,22 @@ fs_status enqueue_depth(fs_handle* h, float* disp, float* depth, cudaStream_t st
   k_depth<<<grid2(L0.W, L0.H), kBlock2, 0, st>>>(L0.v, c, (float)-h->tp[0], (float)-h->tp[1],
                                                  (float)-h->tp[2], disp, depth);
   FS_LAUNCHED("k_depth");
+  return FS_OK;
+}
+
+// The end of a warp (clip + update, Eq. 8-9) in one launch with what follows:
+// the next warp's start (warp + linearise), or after a frame's last warp the
+// triangulation.
+fs_status end_warp(fs_handle* h, int l, int iters, bool next, float* disp, float* depth,
+                   cudaStream_t st) {
+  const bool chain = short_chain(h, l, iters);
+  if (next || l > 0) return run_stage(h, l, next ? FS_STAGE_CLIP_WARP : FS_STAGE_CLIP, 0, st, chain);
+  HostLevel& L0 = h->lv[0];
+  L0.consts_stale = true;
+  FS_LAUNCH("k_clip_depth",
+            launch_clip_depth(L0.v, h->prm.du_max, dev_cam(h->cam[0], L0.fx, L0.fy, L0.cx, L0.cy),
+                              (float)-h->tp[0], (float)-h->tp[1], (float)-h->tp[2], disp, depth,
+                              chain, st));
   return FS_OK;
 }
 
@@ -690,26 +717,23 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
   NvtxRange range(init || cont ? "fs warm solve" : "fs solve");
   fs_status s;
   HostLevel& L0 = h->lv[0];
-  FS_LAUNCH("k_copy_in_s", launch_copy_in_image(I0, L0.v, 0, st));
-  FS_LAUNCH("k_prerotate", launch_prerotate(I1, h->cfield, L0.v, st));
+  FS_LAUNCH("k_prerotate", launch_prerotate(I0, I1, h->cfield, L0.v, st));
   int top = h->L - 1;
   if (init || cont) {   // warm start: the finest level only
     if (finest_wait) FS_CUDA(cudaStreamWaitEvent(st, finest_wait, 0));
     if (cont) {          // from the level's own last u and w
-      FS_LAUNCH("k_continue", launch_continue(L0.v, st));
-      if (h->prm.regularizer == FS_REG_TGV) FS_LAUNCH("k_tgv_reset", launch_tgv_reset(L0.v, st));
+      if ((s = start_level(h, 0, START_CONTINUE, st)) != FS_OK) return s;
     } else {             // from the given disparity, w rebuilt along gamma'
       k_copy_in<<<grid2(L0.W, L0.H), kBlock2, 0, st>>>(init, L0.v.u, L0.W, L0.H, L0.P);
       FS_LAUNCHED("k_copy_in");
       if ((s = run_stage(h, 0, FS_STAGE_WARM, 0, st)) != FS_OK) return s;
+      if ((s = start_level(h, 0, START_GIVEN, st)) != FS_OK) return s;
     }
-    if ((s = run_stage(h, 0, FS_STAGE_TENSOR, 0, st)) != FS_OK) return s;
-    if ((s = run_stage(h, 0, FS_STAGE_WARP, 0, st)) != FS_OK) return s;
     for (int w = 0; w < warps; ++w) {
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w], st));
       if ((s = run_pd(h, 0, iters, st, true)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w + 1], st));
-      if ((s = clip_then_warp(h, 0, iters, w + 1 < warps, st)) != FS_OK) return s;
+      if ((s = end_warp(h, 0, iters, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
     }
     if (h->timing) {
       h->ev_warps = warps;
@@ -718,7 +742,7 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
       h->ev_pending = true;
     }
     if (finest_done) FS_CUDA(cudaEventRecord(finest_done, st));
-    return enqueue_depth(h, disp, depth, st);
+    return FS_OK;
   }
   for (int l = 0; l < top; ++l)
     if ((s = run_stage(h, l, FS_STAGE_DOWNSAMPLE, 0, st)) != FS_OK) return s;
@@ -729,19 +753,12 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     NvtxRange level_range(kLevelNames[l < 8 ? l : 7]);
     HostLevel& L = h->lv[l];
     if (l == 0 && finest_wait) FS_CUDA(cudaStreamWaitEvent(st, finest_wait, 0));
-    if ((s = run_stage(h, l, FS_STAGE_TENSOR, 0, st)) != FS_OK) return s;
-    if (l == top) {
-      FS_LAUNCH("k_zero_state", launch_zero_state(L.v, st));
-      if (h->prm.regularizer == FS_REG_TGV) FS_LAUNCH("k_tgv_reset", launch_tgv_reset(L.v, st));
-    } else if ((s = run_stage(h, l, FS_STAGE_UPSAMPLE, 0, st)) != FS_OK) {
-      return s;
-    }
-    if ((s = run_stage(h, l, FS_STAGE_WARP, 0, st)) != FS_OK) return s;
+    if ((s = start_level(h, l, l == top ? START_ZERO : START_UPSAMPLE, st)) != FS_OK) return s;
     for (int w = 0; w < warps; ++w) {
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w)], st));
       if ((s = run_pd(h, l, iters, st, true)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w) + 1], st));
-      if ((s = clip_then_warp(h, l, iters, w + 1 < warps, st)) != FS_OK) return s;
+      if ((s = end_warp(h, l, iters, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
     }
   }
   if (h->timing) {
@@ -751,7 +768,7 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     h->ev_pending = true;
   }
   if (finest_done) FS_CUDA(cudaEventRecord(finest_done, st));
-  return enqueue_depth(h, disp, depth, st);
+  return FS_OK;
 }
 
 fs_status prepare_timing(fs_handle* h, int warps) {
@@ -998,8 +1015,7 @@ static fs_status enqueue_persist(PersistPlan* P, const std::vector<fs_handle*>& 
   fs_status s;
   for (size_t i = 0; i < hs.size(); ++i) {
     fs_handle* h = hs[i];
-    FS_LAUNCH("k_copy_in_s", launch_copy_in_image(I0[i], h->lv[0].v, 0, st));
-    FS_LAUNCH("k_prerotate", launch_prerotate(I1[i], h->cfield, h->lv[0].v, st));
+    FS_LAUNCH("k_prerotate", launch_prerotate(I0[i], I1[i], h->cfield, h->lv[0].v, st));
     for (int l = 0; l + 1 < h->L; ++l)
       if ((s = run_stage(h, l, FS_STAGE_DOWNSAMPLE, 0, st)) != FS_OK) return s;
   }
@@ -1936,7 +1952,7 @@ extern "C" fs_status fs_stage_prerotate(fs_handle* h, const float* d_I1) {
   if ((s = check_handle(h)) != FS_OK) return s;
   if (!d_I1) return fail(FS_EINVAL, "null input");
   HostLevel& L0 = h->lv[0];
-  FS_LAUNCH("k_prerotate", launch_prerotate(d_I1, h->cfield, L0.v, h->stream));
+  FS_LAUNCH("k_prerotate", launch_prerotate(nullptr, d_I1, h->cfield, L0.v, h->stream));
   return FS_OK;
 }
 

@@ -73,17 +73,16 @@ __global__ void k_mask_to_float(const uint8_t* __restrict__ m, float* __restrict
 
 // Storage-typed kernels, launched through these (the level's storage picks
 // the instantiation).
-cudaError_t launch_prerotate(const float* I1, const float4* field, const LevelView& L0,
-                             cudaStream_t st);
+// (I0 null: I1 only; else also launch_copy_in_image of I0.)
+cudaError_t launch_prerotate(const float* I0, const float* I1, const float4* field,
+                             const LevelView& L0, cudaStream_t st);
 // A dense FP32 image into level L's I0 (which = 0) or I1 (1), with the low
 // part of its rounding to the level's storage (the pyramid's carry).
 cudaError_t launch_copy_in_image(const float* src, const LevelView& L, int which,
                                  cudaStream_t st);
 cudaError_t launch_downsample(const LevelView& F, const LevelView& C, cudaStream_t st);
 cudaError_t launch_upsample(const LevelView& C, const LevelView& F, cudaStream_t st);
-cudaError_t launch_zero_state(const LevelView& L, cudaStream_t st);
 cudaError_t launch_warm_start(const LevelView& L, float du_max, cudaStream_t st);
-cudaError_t launch_continue(const LevelView& L, cudaStream_t st);
 
 // The automatic schedule of `iters` iterations on a level: a footprint
 // (variant), the number of launches and the halo depth (the iterations of
@@ -145,6 +144,18 @@ cudaError_t launch_warp(const LevelView& L, int central, float lam, float eps, i
 cudaError_t launch_clip_warp(const LevelView& L, float du_max, int central, float lam, float eps,
                              int consts, bool chained, cudaStream_t st);
 cudaError_t launch_clip(const LevelView& L, float du_max, bool chained, cudaStream_t st);
+// k_clip of a frame's last warp fused with k_depth (same results).
+cudaError_t launch_clip_depth(const LevelView& L, float du_max, const DevCam& cam, float Cx,
+                              float Cy, float Cz, float* disp, float* depth, bool chained,
+                              cudaStream_t st);
+// The start of level L in one launch: k_tensor, the start state -- zero,
+// upsampled from C, continued from the level's own last u and w, or as it is
+// in the planes -- and k_warp (same results; TGV: v, vbar, q <- 0 too, except
+// for START_GIVEN).
+enum LevelStart { START_ZERO, START_UPSAMPLE, START_CONTINUE, START_GIVEN };
+cudaError_t launch_level_start(int mode, const LevelView& C, const LevelView& L, float beta,
+                               float eta, int precond, int central, float lam, float eps,
+                               int consts, cudaStream_t st);
 cudaError_t launch_tensor_abc(const LevelView& L, float* dst, cudaStream_t st);
 cudaError_t launch_pack_s(const SPlane& src, int storage, float* dst, int W, int H, int P,
                           cudaStream_t st);

@@ -53,7 +53,8 @@ __device__ __forceinline__ float upsample_px(const LevelView& C, const LevelView
     }
     if (den > 0.f) {
       float s = 2.f / den;
-      u = nu * s; wx = nx * s; wy = ny * s;
+      // products of their own: a caller that goes on with w gets the stored bits
+      u = __fmul_rn(nu, s); wx = __fmul_rn(nx, s); wy = __fmul_rn(ny, s);
     }
   }
   F.u[o] = u; F.ubar[o] = u; F.uw[o] = u;
