@@ -467,19 +467,18 @@ PdSchedule pd_plan(const fs_handle* h, int l, int iters) {
   else if (b > 0 && (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0))
     nl = pd_launch_count(iters, b);
   if (L.plan_iters != iters || L.plan_nl != nl) {
-    L.plan = tgv ? tgv_auto(L.v, iters, nl, h->sms) : pd_auto(L.v, iters, nl, h->sms);
+    L.plan = tgv ? tgv_auto(L.v, iters, nl, h->sms) : pd_auto(L.v, iters, nl, h->sms, L.tma_ok);
     L.plan_iters = iters;
     L.plan_nl = nl;
   }
   return L.plan;
 }
 
-// Whether a solve of h runs the TMA-staged footprints on some level.
-bool uses_tma(const fs_handle* h) {
-  if (h->prm.regularizer == FS_REG_TGV || h->prm.block_iters > 0) return false;
+// Whether a solve of h with `iters` iterations a warp runs the TMA-staged footprints on some level.
+bool uses_tma(const fs_handle* h, int iters) {
+  if (h->prm.regularizer == FS_REG_TGV) return false;
   for (int l = 0; l < h->L; ++l)
-    if (h->lv[l].tuned >= 1 && !h->lv[l].auto_best && h->lv[l].tuned_variant == PD_TILE_64_TMA)
-      return true;
+    if (!use_cluster(h, l) && pd_plan(h, l, iters).variant == PD_TILE_64_TMA) return true;
   return false;
 }
 
@@ -578,8 +577,8 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
     pp.launches = nl;
     pp.idle = !ps.skip ? -1 : k == 0 ? iters : 0;
     const int link = k > 0 ? PD_CHAINED : pp.fresh ? PD_CHAIN_START : 0;
-    cudaError_t e = tma ? launch_pd_tma(L.v, out, pp, B, n, link, L.tma[k % 2], h->pd_status,
-                                        h->wait_ns, (h->persist_stall && k == 0) ? 1 : 0, st)
+    cudaError_t e = tma ? launch_pd_tma(L.v, in, out, pp, B, n, link, L.tma[k % 2],
+                                        h->pd_status, h->wait_ns, (h->persist_stall && k == 0) ? 1 : 0, st)
                         : launch_pd(variant, L.v, in, out, pp, B, n, st, link);
     if (e != cudaSuccess)
       return fail(FS_ECUDA, "launch of %s failed: %s", tma ? "k_pd_tma" : "k_pd",
@@ -1503,7 +1502,7 @@ fs_status fs_solve_host(fs_handle* h, const float* h_I0, const float* h_I1, cons
   if (h_disp) FS_CUDA(cudaMemcpyAsync(h_disp, ddisp, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
   if (h_depth) FS_CUDA(cudaMemcpyAsync(h_depth, ddepth, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
   FS_CUDA(cudaStreamSynchronize(h->stream));
-  return uses_tma(h) ? fs_check_waits(h) : FS_OK;
+  return uses_tma(h, iters) ? fs_check_waits(h) : FS_OK;
 }
 
 fs_status fs_destroy(fs_handle* h) {

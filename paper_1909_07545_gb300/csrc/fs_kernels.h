@@ -102,11 +102,16 @@ struct BlockFit {
   int variant, fw, fh, per_sm;
   float t0, b;
   bool skip;
+  // footprints taken in turn by resident CTAs: interior columns, fixed (0:
+  // what the halo leaves), and the microseconds once a launch
+  int iw = 0;
+  float launch = 0.f;
 };
 // The least of the modelled times over n_fit footprints and launch counts.
 PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, int iters,
                           int launches, int sms);
-PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms);    // Huber-TV
+// Huber-TV; tma: the TMA-staged footprints may be chosen
+PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma);
 PdSchedule tgv_auto(const LevelView& L, int iters, int launches, int sms);   // TGV-L1
 // Launches of `iters` iterations at most `depth` each, made even when
 // iters >= 2 so that the ping-pong state ends where it began.
@@ -187,9 +192,25 @@ cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const 
 // level's W x H pixels, pitch P; boxes of 64 x 64 elements, the mask's
 // 80 x 64).
 struct PdTmaMaps {
-  CUtensorMap sx, sy, tau, dinv, sd, step, c0, mask;
-  CUtensorMap u, ubar, p1, p2;
+  CUtensorMap tau, dinv, sd, step, c0;
+  CUtensorMap u, ubar;
+  CUtensorMap sx, sy, p1, p2, mask;
 };
+
+// The footprints of k_pd_tma that may hold FOV pixels: in tile row y the
+// start[y + 1] - start[y] columns from lo[y]; n = 0: all.
+struct PdTmaRows {
+  static constexpr int kMax = 128;
+  int n;
+  unsigned short lo[kMax];
+  int start[kMax + 1];
+};
+// The columns [lo, hi) of a row of tiles, pitch `pitch`, x0 the first one's
+// left edge, fw x fh pixels with the upper edge at line y0, that may hold a
+// pixel of L's FOV ellipse: its half-width at the row's line nearest to its
+// centre, and a pixel more for the rounding.
+void fov_columns(const LevelView& L, int pitch, int x0, int fw, int fh, int tiles_x, int y0,
+                 int& lo, int& hi);
 
 // n (<= B <= 8) primal-dual iterations on the TMA-staged footprints (one
 // resident CTA per SM walking the footprints), the state read through
@@ -197,9 +218,9 @@ struct PdTmaMaps {
 // runs out after wait_ns of global time sets *status to FS_ETIMEOUT;
 // stall = 1 makes the first wait run out (testing aid).  Same results as
 // launch_pd.
-cudaError_t launch_pd_tma(const LevelView& L, const PDState& out, const PDParams& pp, int B,
-                          int n, int chained, const PdTmaMaps& maps, int* status,
-                          unsigned long long wait_ns, int stall, cudaStream_t st);
+cudaError_t launch_pd_tma(const LevelView& L, const PDState& in, const PDState& out,
+                          const PDParams& pp, int B, int n, int chained, const PdTmaMaps& maps,
+                          int* status, unsigned long long wait_ns, int stall, cudaStream_t st);
 // Dynamic shared memory of one k_pd_tma CTA for a storage type.
 size_t pd_tma_smem_bytes(int storage);
 

@@ -265,10 +265,14 @@ int pd_launch_count(int iters, int depth) {
 //   640 x 640  18.7 / 156.4           31.4 / 276.2
 //   1024 x 1024  41.9 / 392           47.5 / 434
 //   2048 x 2048 (50 iterations)  816          1034
+// The TMA-staged footprints' third figure is a launch's own time; they win
+// from where an SM has some six footprints: 100 iterations of 2048 x 2048
+// with a 180-degree FOV 1220 us against 1410-1600 (64 x 32, two per SM), a
+// frame 19.6 ms against 23.7; 1024 x 1024 keeps 64 x 32.
 // Where it saves waves, the footprints outside the FOV are left out: a 2048 x
 // 2048 frame under a 180-degree lens takes 24.0 ms against 27.9.  (With a
 // single wave the test only costs, up to 4 % of a 256 x 256 frame.)
-PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms) {
+PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma) {
   static const BlockFit kFit[] = {
       {PD_TILE_32x16_T256, 32, 16, 1, 1.95f, 0.18f, false},
       {PD_TILE_32x24_T384, 32, 24, 1, 1.85f, 0.185f, false},
@@ -280,8 +284,24 @@ PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms) {
       {PD_TILE_64x48_T768, 64, 48, 1, 3.0f, 0.55f, true},
       {PD_TILE_64_T1024, 64, 64, 1, 4.1f, 0.735f, true},
       {PD_TILE_64x32_T512, 64, 32, 2, 3.2f, 0.67f, true},
+      {PD_TILE_64_TMA, 64, 64, 1, 2.3f, 0.78f, true, 48, 2.8f},
   };
-  return block_schedule(kFit, (int)(sizeof(kFit) / sizeof(kFit[0])), L, iters, launches, sms);
+  return block_schedule(kFit, (int)(sizeof(kFit) / sizeof(kFit[0])) - !tma, L, iters, launches,
+                        sms);
+}
+
+void fov_columns(const LevelView& L, int pitch, int x0, int fw, int fh, int tiles_x, int y0,
+                 int& lo, int& hi) {
+  lo = hi = 0;
+  const double cx = L.fov_cx, cy = L.fov_cy;
+  const double dy = std::max(std::max(y0 - cy, cy - (y0 + fh - 1.0)) - 1.0, 0.0) * L.fov_iy;
+  const double h2 = (double)L.fov_r2 - dy * dy;
+  if (!(h2 >= 0)) return;
+  const double half = std::min(std::sqrt(h2) / L.fov_ix, 1e6) + 1.0;
+  const double a = std::ceil((cx - half - (x0 + fw - 1.0)) / pitch);
+  const double b = std::floor((cx + half - x0) / pitch);
+  lo = (int)std::min(std::max(a, 0.0), (double)tiles_x);
+  hi = std::max((int)std::min(std::max(b + 1.0, 0.0), (double)tiles_x), lo);
 }
 
 PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, int iters,
@@ -295,33 +315,27 @@ PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, in
     if (depth > kMaxDepth) return;
     for (int j = 0; j < n_fit; ++j) {
       const BlockFit& f = fit[j];
-      const int iw = f.fw - 2 * depth, ih = f.fh - 2 * depth;
-      if (iw < 2 || ih < 2) continue;
+      const int bx = f.iw > 0 ? (f.fw - f.iw) / 2 : depth;      // column margin
+      const int iw = f.fw - 2 * bx, ih = f.fh - 2 * depth;
+      if (iw < 2 || ih < 2 || depth > bx) continue;
       const int tx = (L.W + iw - 1) / iw, ty = (L.H + ih - 1) / ih;
       const double seats = (double)f.per_sm * sms;
       double waves = std::ceil((double)tx * ty / seats);
-      const double us1 = nl * (f.t0 + f.b * iters / nl);
       bool skip = false;
       if (f.skip && waves > 1.0 && nl > 1) {
-        // the footprints that reach the FOV ellipse, row by row of tiles: those
-        // within its half-width at the row's nearest line to the centre
-        double active = 0;
+        double active = 0;           // footprints that may hold FOV pixels
         for (int y = 0; y < ty; ++y) {
-          const double y0 = (double)y * ih - depth, y1 = y0 + f.fh - 1;
-          const double dy = std::max(std::max(y0 - L.fov_cy, L.fov_cy - y1), 0.0) * L.fov_iy;
-          const double h2 = (double)L.fov_r2 - dy * dy;
-          if (!(h2 >= 0)) continue;
-          const double half = std::min(std::sqrt(h2) / L.fov_ix, 1e6);
-          const double lo = std::floor((L.fov_cx - half - (f.fw - 1) + depth) / iw);
-          const double hi = std::floor((L.fov_cx + half + depth) / iw);
-          active += std::max(0.0, std::min(hi, tx - 1.0) - std::max(lo, 0.0) + 1.0);
+          int lo, hi;
+          fov_columns(L, iw, -bx, f.fw, f.fh, tx, y * ih - depth, lo, hi);
+          active += hi - lo;
         }
         const double left = std::max(std::ceil(active / seats), 1.0);
         skip = left < waves;
         if (skip) waves = left;
       }
-      if (us1 * waves < best_us) {
-        best_us = us1 * waves;
+      const double us = nl * (f.launch + waves * (f.t0 + f.b * iters / nl));
+      if (us < best_us) {
+        best_us = us;
         best = PdSchedule{f.variant, nl, depth, skip};
       }
     }

@@ -24,9 +24,9 @@
 // such pixels (no mask bit, all constants and state 0).
 //
 // Synchronisation.  One mbarrier: the leader thread arms it with the bytes
-// of a footprint (arrive.expect_tx) and issues the twelve copies; every
+// of a footprint (arrive.expect_tx), twelve warps issue a copy each; every
 // thread waits on its phase (try_wait.parity) before reading the planes.
-// The planes of the next footprint are requested only after a CTA barrier
+// The planes of the next footprint are requested only after the CTA barrier
 // that follows every thread's reads of the current one.  Every wait is
 // bounded by wait_ns of global time; a wait that runs out sets *status to
 // FS_ETIMEOUT and the CTA returns.
@@ -110,31 +110,18 @@ __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// The leader's requests for footprint `tile`: the per-warp constants (and
-// the mask), then, when `state`, the primal-dual state of the input set.
+// The twelve copies of a footprint, in the order of PdTmaMaps and of the
+// shared-memory planes; one warp requests each.
+constexpr int kCopies = 12;
+__device__ __forceinline__ bool is_state(int k) { return k == 5 || k == 6 || k == 9 || k == 10; }
+
 template <int S>
 __device__ __forceinline__ void request(const PdTmaMaps& m, unsigned char* smem, uint32_t bar,
-                                        int tile, int tiles_x, int IH, int B, bool consts,
-                                        bool state) {
+                                        int k, int bx, int by, int IH, int B) {
   using Lay = TmaLayout<S>;
-  const int bx = tile % tiles_x, by = tile / tiles_x;
-  const int x = bx * kIW - kXM, y = by * IH - B;
-  if (consts) {
-    tma_load(smem_addr(smem + Lay::tau), &m.tau, x, y, bar);
-    tma_load(smem_addr(smem + Lay::dinv), &m.dinv, x, y, bar);
-    tma_load(smem_addr(smem + Lay::sd), &m.sd, x, y, bar);
-    tma_load(smem_addr(smem + Lay::step), &m.step, x, y, bar);
-    tma_load(smem_addr(smem + Lay::c0), &m.c0, x, y, bar);
-    tma_load(smem_addr(smem + Lay::sx), &m.sx, x, y, bar);
-    tma_load(smem_addr(smem + Lay::sy), &m.sy, x, y, bar);
-    tma_load(smem_addr(smem + Lay::mask), &m.mask, bx * kIW - kMaskOff, y, bar);
-  }
-  if (state) {
-    tma_load(smem_addr(smem + Lay::u), &m.u, x, y, bar);
-    tma_load(smem_addr(smem + Lay::ub), &m.ubar, x, y, bar);
-    tma_load(smem_addr(smem + Lay::p1), &m.p1, x, y, bar);
-    tma_load(smem_addr(smem + Lay::p2), &m.p2, x, y, bar);
-  }
+  const size_t dst = k < 7 ? k * Lay::f32 : Lay::sx + (k - 7) * Lay::sp;   // the mask follows p2
+  tma_load(smem_addr(smem + dst), reinterpret_cast<const CUtensorMap*>(&m) + k,
+           bx * kIW - (k == 11 ? kMaskOff : kXM), by * IH - B, bar);
 }
 
 // A staged storage-typed value (FP16 / BF16 converted to float).
@@ -148,58 +135,77 @@ __device__ __forceinline__ float sval(const unsigned char* plane, int k) {
 
 }  // namespace
 
-// n_iters (<= B <= 8) iterations on every footprint of the level; the state
-// is read (through the copies in `maps`) from one buffer set and written to
-// `out`.  chained (pd_tile): PD_CHAINED requests the first footprint's
-// constants before the wait for the preceding launch and its state after,
-// PD_CHAIN_START waits first.  stall: testing aid, the first wait never completes.
+// n_iters (<= B <= 8) iterations on the level's footprints --
+// those of `rows` where rows.n > 0 (the others hold no FOV pixel; pp.idle),
+// else all; the state is read (through the copies in `maps`) from the buffer
+// set `in` and written to `out`.  chained (pd_tile): PD_CHAINED requests the
+// first footprint's constants before the wait for the preceding launch and
+// its state after, PD_CHAIN_START waits first.  stall: testing aid, the
+// first wait never completes.
+//
+// Bound by the iterations, 1450-1700 clock cycles each, and by what lies
+// between two footprints: 3800 cycles, the 1400 shared-memory wavefronts of
+// the reads among them, against 7000 when one thread requested all the copies
+// and four barriers kept the stores, the reads and the requests apart.  2048
+// x 2048, 100 iterations: 14.9 us each against 16.4, 12.2 without the
+// footprints outside a 180-degree FOV (19.3 on 64 x 64 footprints of k_pd).
 template <int S, bool ACC>
 __global__ void __launch_bounds__(kFW * kNY, 1)
-k_pd_tma(LevelView L, PDState out, PDParams pp, int B, int n_iters, int chained,
-         const __grid_constant__ PdTmaMaps maps, int* status, unsigned long long wait_ns,
-         int stall) {
+k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, int chained,
+         const __grid_constant__ PdTmaMaps maps, const __grid_constant__ PdTmaRows rows,
+         int* status, unsigned long long wait_ns, int stall) {
   using Lay = TmaLayout<S>;
   extern __shared__ __align__(128) unsigned char smem[];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const bool leader = tx == 0 && ty == 0;
+  // the copy this thread requests, -1: none
+  const int copy = (tx & 31) == 0 && 2 * ty + (tx >> 5) < kCopies ? 2 * ty + (tx >> 5) : -1;
   const int IH = kFH - 2 * B;
   const int tiles_x = (L.W + kIW - 1) / kIW;
-  const int ntiles = tiles_x * ((L.H + IH - 1) / IH);
+  const int all_tiles = tiles_x * ((L.H + IH - 1) / IH);
+  const int ntiles = rows.n > 0 ? rows.start[rows.n] : all_tiles;
   float(*s_ub)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_ub);
   float(*s_t1)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_t1);
   float(*s_t2)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_t2);
   const uint32_t bar = smem_addr(smem + Lay::bar);
+  volatile int* s_late = reinterpret_cast<volatile int*>(smem + Lay::bar + 16);
+
+  // footprint t's place; by: a row at or before it (only ever moves down)
+  auto column = [&](int t, int& by) {
+    if (rows.n == 0) {
+      by = t / tiles_x;
+      return t - by * tiles_x;
+    }
+    while (t >= rows.start[by + 1]) ++by;
+    return rows.lo[by] + t - rows.start[by];
+  };
 
   // the next launch of the chain may be scheduled once every CTA of this one
   // is resident (it waits for this grid's completion before its state); for
   // the first of a chain once the constants are complete
   if (chained == PD_CHAIN_START) cudaGridDependencySynchronize();
   if (chained) cudaTriggerProgrammaticLaunchCompletion();
-  int tile = blockIdx.x;
+  int tile = blockIdx.x, by = 0, bx = tile < ntiles ? column(tile, by) : 0;
   if (leader) {
     mbar_init(bar, 1);
-    if (tile < ntiles) {
-      mbar_expect_tx(bar, Lay::tx + (stall ? 16u : 0u));
-      request<S>(maps, smem, bar, tile, tiles_x, IH, B, true, false);
-    }
+    *s_late = 0;
+    if (tile < ntiles) mbar_expect_tx(bar, Lay::tx + (stall ? 16u : 0u));
   }
-  if (chained == PD_CHAINED) cudaGridDependencySynchronize();
-  if (leader && tile < ntiles) request<S>(maps, smem, bar, tile, tiles_x, IH, B, false, true);
   __syncthreads();
+  if (copy >= 0 && tile < ntiles && !is_state(copy))
+    request<S>(maps, smem, bar, copy, bx, by, IH, B);
+  if (chained == PD_CHAINED) cudaGridDependencySynchronize();
+  if (copy >= 0 && tile < ntiles && is_state(copy))
+    request<S>(maps, smem, bar, copy, bx, by, IH, B);
 
   unsigned parity = 0;
-  for (; tile < ntiles; tile += gridDim.x) {
-    bool late = false;
+  while (tile < ntiles) {
     const unsigned long long t0 = global_ns();
     while (!mbar_try_wait(bar, parity)) {
       if (global_ns() - t0 > wait_ns) {
-        late = true;
+        *s_late = 1;
         break;
       }
-    }
-    if (__syncthreads_or(late)) {
-      if (leader) atomicCAS(status, 0, (int)FS_ETIMEOUT);
-      return;
     }
     parity ^= 1u;
 
@@ -207,45 +213,51 @@ k_pd_tma(LevelView L, PDState out, PDParams pp, int B, int n_iters, int chained,
     float u[kR], ub[kR], p1[kR], p2[kR];
     PxConst c[kR];
     unsigned mb = 0;
-    {
-      // (outside the level the copies read zeros: the constants of k_pd's
-      // all-zero inputs, except dinv = 0 instead of 1, which only scales a
-      // dual that is 0 there and stays 0)
+    // (outside the level the copies read zeros: the constants of k_pd's
+    // all-zero inputs, except dinv = 0 instead of 1, which only scales a
+    // dual that is 0 there and stays 0)
 #pragma unroll
-      for (int r = 0; r < kR; ++r) {
-        const int k = (ty * kR + r) * kFW + tx;
-        auto f32 = [&](size_t plane) { return reinterpret_cast<const float*>(smem + plane)[k]; };
-        c[r].tau = f32(Lay::tau);
-        c[r].dinv = f32(Lay::dinv);
-        c[r].sd = f32(Lay::sd);
-        c[r].step = f32(Lay::step);
-        c[r].c0 = f32(Lay::c0);
-        c[r].sx = sval<S>(smem + Lay::sx, k);
-        c[r].sy = sval<S>(smem + Lay::sy, k);
-        u[r] = f32(Lay::u);
-        ub[r] = f32(Lay::ub);
-        p1[r] = sval<S>(smem + Lay::p1, k);
-        p2[r] = sval<S>(smem + Lay::p2, k);
-        mb |= (unsigned)smem[Lay::mask + (ty * kR + r) * kMaskW + tx + (kMaskOff - kXM)]
-              << (3 * r);
-      }
-      __syncthreads();            // every thread has read the staged planes
-      const int next = tile + (int)gridDim.x;
-      if (leader && next < ntiles) {
-        // order the reads above before the copies that overwrite the planes
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(bar, Lay::tx);
-        request<S>(maps, smem, bar, next, tiles_x, IH, B, true, true);
-      }
+    for (int r = 0; r < kR; ++r) {
+      const int k = (ty * kR + r) * kFW + tx;
+      auto f32 = [&](size_t plane) { return reinterpret_cast<const float*>(smem + plane)[k]; };
+      c[r].tau = f32(Lay::tau);
+      c[r].dinv = f32(Lay::dinv);
+      c[r].sd = f32(Lay::sd);
+      c[r].step = f32(Lay::step);
+      c[r].c0 = f32(Lay::c0);
+      c[r].sx = sval<S>(smem + Lay::sx, k);
+      c[r].sy = sval<S>(smem + Lay::sy, k);
+      u[r] = f32(Lay::u);
+      ub[r] = f32(Lay::ub);
+      p1[r] = sval<S>(smem + Lay::p1, k);
+      p2[r] = sval<S>(smem + Lay::p2, k);
+      mb |= (unsigned)smem[Lay::mask + (ty * kR + r) * kMaskW + tx + (kMaskOff - kXM)]
+            << (3 * r);
     }
 #pragma unroll
     for (int r = 0; r < kR; ++r) s_ub[ty * kR + r][tx] = ub[r];
-    __syncthreads();
+    // one barrier: every thread has read the staged planes, ubar is in place
+    // for the neighbours, and whether every pixel of the footprint lies in
+    // the level with all three mask bits set (outside it the mask reads 0).
+    // (s_ub: the last footprint's iterations ended with a barrier.)
+    const bool full = __syncthreads_and(mb == 07777u);
+    if (*s_late) {
+      if (leader) atomicCAS(status, 0, (int)FS_ETIMEOUT);
+      return;
+    }
+    if (n_iters == 0) __syncthreads();   // s_late and s_ub as if iterations followed
+    const int next = tile + (int)gridDim.x;
+    int nby = by;
+    const int nbx = next < ntiles ? column(next, nby) : 0;
+    if (copy >= 0 && next < ntiles) {
+      if (leader) mbar_expect_tx(bar, Lay::tx);
+      // order the reads above before the copies that overwrite the planes
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      request<S>(maps, smem, bar, copy, nbx, nby, IH, B);
+    }
 
-    // every pixel of the footprint in the level with all three mask bits
-    // set (pixels outside the level were filled with mask 0)
     float theta = pp.theta;
-    if (__syncthreads_and(mb == 07777u))
+    if (full)
       pd_iterate_rows<kFW, kNY, kR, ACC, false>(pp, n_iters, tx, ty, mb, c, u, ub, p1, p2,
                                                 theta, s_ub, s_t1, s_t2);
     else
@@ -253,29 +265,41 @@ k_pd_tma(LevelView L, PDState out, PDParams pp, int B, int n_iters, int chained,
                                                theta, s_ub, s_t1, s_t2);
 
     // the interior back to global memory
-    const int bx = tile % tiles_x, by = tile / tiles_x;
     const int gx = bx * kIW - kXM + tx;
-    if (tx < kXM || tx >= kXM + kIW || gx >= L.W) continue;
+    if (tx >= kXM && tx < kXM + kIW && gx < L.W) {
 #pragma unroll
-    for (int r = 0; r < kR; ++r) {
-      const int fy = ty * kR + r;
-      const int gy = by * IH - B + fy;
-      if (fy < B || fy >= kFH - B || gy >= L.H) continue;
-      const size_t i = (size_t)gy * L.P + gx;
-      out.u[i] = u[r];
-      out.ubar[i] = ub[r];
-      sst<S>(out.p1, i, p1[r]);
-      sst<S>(out.p2, i, p2[r]);
+      for (int r = 0; r < kR; ++r) {
+        const int fy = ty * kR + r;
+        const int gy = by * IH - B + fy;
+        if (fy < B || fy >= kFH - B || gy >= L.H) continue;
+        const size_t i = (size_t)gy * L.P + gx;
+        out.u[i] = u[r];
+        out.ubar[i] = ub[r];
+        sst<S>(out.p1, i, p1[r]);
+        sst<S>(out.p2, i, p2[r]);
+      }
     }
+    tile = next;
+    bx = nbx;
+    by = nby;
+  }
+
+  // the first launch of a warp: all its iterations on the footprints left out
+  if (rows.n == 0 || pp.idle <= 0) return;
+  for (int t = blockIdx.x; t < all_tiles; t += (int)gridDim.x) {
+    const int y = t / tiles_x, x = t - y * tiles_x;
+    const int k = x - rows.lo[y];
+    if (k >= 0 && k < rows.start[y + 1] - rows.start[y]) continue;
+    pd_idle<kFW, kNY, kR, S, ACC>(L, in, pp, kXM, B, x * kIW - kXM, y * IH - B, tx, ty);
   }
 }
 
 namespace {
 
 template <int S, bool ACC>
-cudaError_t launch_tma_t(const LevelView& L, const PDState& out, const PDParams& pp, int B,
-                         int n, int chained, const PdTmaMaps& maps, int* status,
-                         unsigned long long wait_ns, int stall, cudaStream_t st) {
+cudaError_t launch_tma_t(const LevelView& L, const PDState& in, const PDState& out,
+                         const PDParams& pp, int B, int n, int chained, const PdTmaMaps& maps,
+                         int* status, unsigned long long wait_ns, int stall, cudaStream_t st) {
   using Lay = TmaLayout<S>;
   static bool configured = false;
   static int sms = 0;
@@ -291,7 +315,19 @@ cudaError_t launch_tma_t(const LevelView& L, const PDState& out, const PDParams&
     configured = true;
   }
   const int IH = kFH - 2 * B;
-  const int ntiles = ((L.W + kIW - 1) / kIW) * ((L.H + IH - 1) / IH);
+  const int tiles_x = (L.W + kIW - 1) / kIW, tiles_y = (L.H + IH - 1) / IH;
+  PdTmaRows rows{};
+  int ntiles = tiles_x * tiles_y;
+  if (pp.idle >= 0 && tiles_y <= PdTmaRows::kMax) {
+    rows.n = tiles_y;
+    for (int y = 0; y < tiles_y; ++y) {
+      int lo = 0, hi = 0;
+      fov_columns(L, kIW, -kXM, kFW, kFH, tiles_x, y * IH - B, lo, hi);
+      rows.lo[y] = (unsigned short)lo;
+      rows.start[y + 1] = rows.start[y] + (hi - lo);
+    }
+    ntiles = std::max(rows.start[tiles_y], 1);
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::min(ntiles, sms), 1, 1);
   cfg.blockDim = dim3(kFW, kNY, 1);
@@ -302,7 +338,7 @@ cudaError_t launch_tma_t(const LevelView& L, const PDState& out, const PDParams&
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k_pd_tma<S, ACC>, L, out, pp, B, n, chained, maps,
+  return cudaLaunchKernelEx(&cfg, k_pd_tma<S, ACC>, L, in, out, pp, B, n, chained, maps, rows,
                             status, wait_ns, stall);
 }
 
@@ -316,23 +352,23 @@ size_t pd_tma_smem_bytes(int storage) {
   }
 }
 
-cudaError_t launch_pd_tma(const LevelView& L, const PDState& out, const PDParams& pp, int B,
-                          int n, int chained, const PdTmaMaps& maps, int* status,
-                          unsigned long long wait_ns, int stall, cudaStream_t st) {
+cudaError_t launch_pd_tma(const LevelView& L, const PDState& in, const PDState& out,
+                          const PDParams& pp, int B, int n, int chained, const PdTmaMaps& maps,
+                          int* status, unsigned long long wait_ns, int stall, cudaStream_t st) {
   if (B < 1 || B > kXM || n < 0 || n > B || L.W < 1 || L.H < 1) return cudaErrorInvalidValue;
   if (pp.sched) {
     if (L.st != ST_F32) return cudaErrorInvalidValue;
-    return launch_tma_t<ST_F32, true>(L, out, pp, B, n, chained, maps, status, wait_ns, stall, st);
+    return launch_tma_t<ST_F32, true>(L, in, out, pp, B, n, chained, maps, status, wait_ns, stall, st);
   }
   switch (L.st) {
     case ST_F16:
-      return launch_tma_t<ST_F16, false>(L, out, pp, B, n, chained, maps, status, wait_ns, stall,
+      return launch_tma_t<ST_F16, false>(L, in, out, pp, B, n, chained, maps, status, wait_ns, stall,
                                          st);
     case ST_BF16:
-      return launch_tma_t<ST_BF16, false>(L, out, pp, B, n, chained, maps, status, wait_ns,
+      return launch_tma_t<ST_BF16, false>(L, in, out, pp, B, n, chained, maps, status, wait_ns,
                                           stall, st);
     default:
-      return launch_tma_t<ST_F32, false>(L, out, pp, B, n, chained, maps, status, wait_ns, stall,
+      return launch_tma_t<ST_F32, false>(L, in, out, pp, B, n, chained, maps, status, wait_ns, stall,
                                          st);
   }
 }

@@ -200,17 +200,17 @@ __device__ __forceinline__ bool outside_fov(const LevelView& L, int x, int y, in
   return dx * dx + dy * dy > L.fov_r2;
 }
 
-// The warp's pp.idle iterations, in place, on the interior pixels of a
-// footprint without a FOV pixel: they move on their own (no difference leaves
+// The warp's pp.idle iterations, in place, on the interior pixels (margins BX
+// columns and B rows) of a footprint without a FOV pixel: they move on their own (no difference leaves
 // them, tau = 0), and not at all where p = 0 and ubar = u, as every warp of a
 // solve starts.  p is rounded to the storage where each of the warp's
 // launches ends.
 template <int FW, int NY, int R, int S, bool ACC>
 __device__ __forceinline__ void pd_idle(const LevelView& L, const PDState& io,
-                                        const PDParams& pp, int B, int ox, int oy, int tx,
-                                        int ty) {
+                                        const PDParams& pp, int BX, int B, int ox, int oy,
+                                        int tx, int ty) {
   const int gx = ox + tx;
-  if (gx < 0 || gx >= L.W || tx < B || tx >= FW - B) return;
+  if (gx < 0 || gx >= L.W || tx < BX || tx >= FW - BX) return;
 #pragma unroll 1
   for (int r = 0; r < R; ++r) {
     const int fy = ty * R + r, gy = oy + fy;
@@ -290,7 +290,7 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
   if constexpr (IDLE) {
     if (outside_fov(L, ox, oy, FW, FH)) {
       if (chained && (pp.idle > 0 || (bx == 0 && by == 0))) cudaGridDependencySynchronize();
-      if (pp.idle > 0) pd_idle<FW, NY, R, S, ACC>(L, in, pp, B, ox, oy, tx, ty);
+      if (pp.idle > 0) pd_idle<FW, NY, R, S, ACC>(L, in, pp, B, B, ox, oy, tx, ty);
       return;
     }
   }

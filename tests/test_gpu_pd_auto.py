@@ -74,6 +74,33 @@ def test_footprints_outside_the_fov(W, H, iters, prm):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("prm", [dict(), dict(precond=0, accel_gamma=0.3), dict(storage="f16"),
+                                 dict(storage="bf16")])
+@pytest.mark.parametrize("W, H, iters", [(2048, 1701, 13), (2251, 2048, 12)])
+def test_large_levels_and_footprints_outside_the_fov(W, H, iters, prm):
+    # the sizes at which the TMA-staged footprints are chosen, an off-centre
+    # FOV, arbitrary state outside it
+    cam = dict(model="equidistant", fx=450.0, fy=520.0, cx=900.3, cy=1020.8, k=[0] * 4, fov_deg=170.0)
+    rng = np.random.default_rng(6)
+    p = dict(I0=rng.random((H, W)), I1=rng.random((H, W)), cam0=cam, cam1=dict(cam), R=np.eye(3),
+             t=np.array([-0.1, 0.0, 0.0]), levels=1)
+    state = {"U": rng.uniform(-1, 1, (H, W)), "UBAR": rng.uniform(-1, 1, (H, W)),
+             "P": rng.uniform(-0.9, 0.9, (2, H, W))}
+    outs = []
+    for choice in (-1, 30):
+        s = make_solver(p, levels=1, **prm)
+        s.set_schedule([choice])
+        s.solve(p["I0"], p["I1"], 1, 2)
+        for b, v in state.items():
+            s.write(0, b, v)
+        s.stage(0, "PD", iters)
+        s.check_waits()
+        outs.append([np64(s.read(0, b)) for b in state])
+        s.close()
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
 TGV = ("U", "UBAR", "V", "VBAR", "P", "Q")
 
 
