@@ -642,7 +642,8 @@ fs_status run_stage(fs_handle* h, int l, int stage, int count, cudaStream_t st,
     case FS_STAGE_CLIP_WARP:
       FS_LAUNCH("k_clip_warp", launch_clip_warp(L.v, h->prm.du_max,
                                                 h->prm.deriv == FS_DERIV_CENTRAL, h->prm.lambda,
-                                                h->prm.huber_eps, consts, chain, st));
+                                                h->prm.huber_eps, consts, !L.consts_stale, chain,
+                                                st));
       L.consts_stale = false;
       return FS_OK;
     case FS_STAGE_WARM:

@@ -145,9 +145,10 @@ cudaError_t launch_warp(const LevelView& L, int central, float lam, float eps, i
 // k_clip of one warp fused with k_warp of the next (same results).  chained:
 // a programmatic dependent launch behind the warp's iterations, which waits
 // for them before it reads anything they or the last warp start wrote; so for
-// k_clip.
+// k_clip.  keep: the constants are the level's current ones but for I_u,
+// rho0 and u_w, and those that follow from sigma alone are left as they are.
 cudaError_t launch_clip_warp(const LevelView& L, float du_max, int central, float lam, float eps,
-                             int consts, bool chained, cudaStream_t st);
+                             int consts, bool keep, bool chained, cudaStream_t st);
 cudaError_t launch_clip(const LevelView& L, float du_max, bool chained, cudaStream_t st);
 // k_clip of a frame's last warp fused with k_depth (same results).
 cudaError_t launch_clip_depth(const LevelView& L, float du_max, const DevCam& cam, float Cx,

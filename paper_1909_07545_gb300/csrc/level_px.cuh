@@ -171,15 +171,17 @@ __device__ __forceinline__ void warp_px(const LevelView& L, int x, int y, size_t
 // ------------------------------------------------------------ clip + update
 // du = clamp(u - u_w, +-du_max); u_{w+1} = u_w + du; w += du g (Algorithm 1,
 // Eq. 8-9).  The primal state continues from u_{w+1}.
+__device__ __forceinline__ float clip_u(float u, float uw, float2 g, float du_max, float2& w) {
+  const float du = fminf(fmaxf(__fsub_rn(u, uw), -du_max), du_max);
+  w = make_float2(fmaf(du, g.x, w.x), fmaf(du, g.y, w.y));
+  return __fadd_rn(uw, du);
+}
+
 template <bool CG>
 __device__ __forceinline__ float clip_px(const LevelView& L, size_t i, float du_max,
                                          float2& w) {
-  float uw = ldf<CG>(L.uw + i);
-  float du = fminf(fmaxf(__fsub_rn(ldf<CG>(L.u + i), uw), -du_max), du_max);
-  float2 g = ldf2<CG>(L.g + i);
   w = ldf2<CG>(L.w + i);
-  w = make_float2(fmaf(du, g.x, w.x), fmaf(du, g.y, w.y));
-  return __fadd_rn(uw, du);
+  return clip_u(ldf<CG>(L.u + i), ldf<CG>(L.uw + i), ldf2<CG>(L.g + i), du_max, w);
 }
 
 }  // namespace fs
