@@ -534,7 +534,8 @@ fs_status ensure_schedule(fs_handle* h, int iters) {
 
 // chain: the launch before on the stream is this library's warp start of the
 // level (the first launch may then be a programmatic dependent one).
-fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = false) {
+fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = false,
+                 int warp = 0) {
   HostLevel& L = h->lv[l];
   PDParams pp{h->prm.lambda, h->prm.huber_eps, h->prm.theta};
   if (h->prm.accel_gamma > 0) {
@@ -576,7 +577,10 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
     pp.k0 = done;
     pp.launches = nl;
     pp.idle = !ps.skip ? -1 : k == 0 ? iters : 0;
-    const int link = k > 0 ? PD_CHAINED : pp.fresh ? PD_CHAIN_START : 0;
+    const int link = k > 0       ? PD_CHAINED
+                     : !pp.fresh ? 0
+                     : warp > 0  ? PD_CHAIN_WARP
+                                 : PD_CHAIN_START;
     cudaError_t e = tma ? launch_pd_tma(L.v, in, out, pp, B, n, link, L.tma[k % 2],
                                         h->pd_status, h->wait_ns, (h->persist_stall && k == 0) ? 1 : 0, st)
                         : launch_pd(variant, L.v, in, out, pp, B, n, st, link);
@@ -731,7 +735,7 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     }
     for (int w = 0; w < warps; ++w) {
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w], st));
-      if ((s = run_pd(h, 0, iters, st, true)) != FS_OK) return s;
+      if ((s = run_pd(h, 0, iters, st, true, w)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w + 1], st));
       if ((s = end_warp(h, 0, iters, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
     }
@@ -756,7 +760,7 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     if ((s = start_level(h, l, l == top ? START_ZERO : START_UPSAMPLE, st)) != FS_OK) return s;
     for (int w = 0; w < warps; ++w) {
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w)], st));
-      if ((s = run_pd(h, l, iters, st, true)) != FS_OK) return s;
+      if ((s = run_pd(h, l, iters, st, true, w)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w) + 1], st));
       if ((s = end_warp(h, l, iters, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
     }

@@ -183,7 +183,7 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   // the next launch of the chain may be scheduled once every CTA of this one
   // is resident (it waits for this grid's completion before its state); for
   // the first of a chain once the constants are complete
-  if (chained == PD_CHAIN_START) cudaGridDependencySynchronize();
+  if (chained >= PD_CHAIN_START) cudaGridDependencySynchronize();
   if (chained) cudaTriggerProgrammaticLaunchCompletion();
   int tile = blockIdx.x, by = 0, bx = tile < ntiles ? column(tile, by) : 0;
   if (leader) {

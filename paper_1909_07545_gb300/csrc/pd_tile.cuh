@@ -20,7 +20,7 @@
 namespace fs {
 
 // How a primal-dual launch follows the kernel before it (pd_tile).
-enum PdChain { PD_CHAINED = 1, PD_CHAIN_START = 2 };
+enum PdChain { PD_CHAINED = 1, PD_CHAIN_START = 2, PD_CHAIN_WARP = 3 };
 
 // The n_iters iterations of pd_tile on a thread's R rows (state in
 // registers, neighbours through shared memory); MASKED as in px_dual.
@@ -301,7 +301,8 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
   // the constants are complete, which the next one reads without waiting.
   if constexpr (CL2 && !CG)
     if (chained == PD_CHAIN_START) cudaGridDependencySynchronize();
-  if (chained) cudaTriggerProgrammaticLaunchCompletion();
+  if (chained && !(CL2 && !CG && chained == PD_CHAIN_WARP))
+    cudaTriggerProgrammaticLaunchCompletion();
 
   float u[R], ub[R], p1[R], p2[R];
   PxConst c[R];
@@ -324,10 +325,9 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const unsigned i = idx[r];
-      const float sx = sld_m<S, CG>(L.sx, i), sy = sld_m<S, CG>(L.sy, i);
-      const float tau = ldf<CG>(L.tau + i), dinv = ldf<CL2>(L.dinv + i);
-      const float sd = ldf<CL2>(L.sd + i), step = ldf<CL2>(L.step + i);
-      const float c0 = ldf<CL2>(L.c0 + i);
+      const float sx = sld_m<S, CL2>(L.sx, i), sy = sld_m<S, CL2>(L.sy, i);
+      const float tau = ldf<CL2>(L.tau + i), dinv = ldf<CL2>(L.dinv + i);
+      const float sd = ldf<CL2>(L.sd + i);
       const unsigned m8 = L.mask[i];
       // outside the level: the constants of all-zero inputs (px_make)
       c[r].sx = ok[r] ? sx : 0.f;
@@ -335,9 +335,19 @@ __device__ __forceinline__ void pd_tile(const LevelView& L, const PDState& in,
       c[r].tau = ok[r] ? tau : 0.f;
       c[r].dinv = ok[r] ? dinv : 1.f;
       c[r].sd = ok[r] ? sd : 0.f;
+      mb |= (ok[r] ? m8 : 0u) << (3 * r);
+    }
+    if constexpr (CL2 && !CG) {
+      if (chained == PD_CHAIN_WARP) {
+        cudaGridDependencySynchronize();
+        cudaTriggerProgrammaticLaunchCompletion();
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const float step = ldf<CL2>(L.step + idx[r]), c0 = ldf<CL2>(L.c0 + idx[r]);
       c[r].step = ok[r] ? step : 0.f;
       c[r].c0 = ok[r] ? c0 : 0.f;
-      mb |= (ok[r] ? m8 : 0u) << (3 * r);
     }
   } else {
     PxRaw raw[R];
