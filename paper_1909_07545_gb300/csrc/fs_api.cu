@@ -674,6 +674,29 @@ fs_status start_level(fs_handle* h, int l, int mode, cudaStream_t st) {
   return FS_OK;
 }
 
+// Both images of a cold solve into the finest level and down the pyramid.
+fs_status enqueue_pyramid(fs_handle* h, const float* I0, const float* I1, cudaStream_t st) {
+  const LevelView* v[kMaxLevels];
+  for (int l = 0; l < h->L; ++l) {
+    v[l] = &h->lv[l].v;
+    h->lv[l].consts_stale = true;
+  }
+  // in one launch where its CTAs run in about one go (four on each SM); on
+  // larger images the launches count less than the threads that idle on the
+  // coarse levels (256 x 256: 488.5 -> 485.4 us a frame, 800 x 800: 1596 ->
+  // 1601, 2048 x 2048: 19.43 -> 19.53 ms)
+  int n = 1;
+  if (pyramid_blocks(*v[0]) <= 4 * h->sms) {
+    n = std::min(h->L, kPyramidLevels);
+    FS_LAUNCH("k_pyramid", launch_pyramid(I0, I1, h->cfield, v, n, st));
+  } else {
+    FS_LAUNCH("k_prerotate", launch_prerotate(I0, I1, h->cfield, *v[0], st));
+  }
+  for (int l = n - 1; l + 1 < h->L; ++l)
+    FS_LAUNCH("k_downsample", launch_downsample(h->lv[l].v, h->lv[l + 1].v, st));
+  return FS_OK;
+}
+
 fs_status enqueue_depth(fs_handle* h, float* disp, float* depth, cudaStream_t st) {
   HostLevel& L0 = h->lv[0];
   DevCam c = dev_cam(h->cam[0], L0.fx, L0.fy, L0.cx, L0.cy);
@@ -721,9 +744,9 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
   NvtxRange range(init || cont ? "fs warm solve" : "fs solve");
   fs_status s;
   HostLevel& L0 = h->lv[0];
-  FS_LAUNCH("k_prerotate", launch_prerotate(I0, I1, h->cfield, L0.v, st));
   int top = h->L - 1;
   if (init || cont) {   // warm start: the finest level only
+    FS_LAUNCH("k_prerotate", launch_prerotate(I0, I1, h->cfield, L0.v, st));
     if (finest_wait) FS_CUDA(cudaStreamWaitEvent(st, finest_wait, 0));
     if (cont) {          // from the level's own last u and w
       if ((s = start_level(h, 0, START_CONTINUE, st)) != FS_OK) return s;
@@ -748,8 +771,7 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     if (finest_done) FS_CUDA(cudaEventRecord(finest_done, st));
     return FS_OK;
   }
-  for (int l = 0; l < top; ++l)
-    if ((s = run_stage(h, l, FS_STAGE_DOWNSAMPLE, 0, st)) != FS_OK) return s;
+  if ((s = enqueue_pyramid(h, I0, I1, st)) != FS_OK) return s;
   for (int l = top; l >= 0; --l) {
     static const char* kLevelNames[] = {"fs level 0", "fs level 1", "fs level 2",
                                         "fs level 3", "fs level 4", "fs level 5",
@@ -1019,9 +1041,7 @@ static fs_status enqueue_persist(PersistPlan* P, const std::vector<fs_handle*>& 
   fs_status s;
   for (size_t i = 0; i < hs.size(); ++i) {
     fs_handle* h = hs[i];
-    FS_LAUNCH("k_prerotate", launch_prerotate(I0[i], I1[i], h->cfield, h->lv[0].v, st));
-    for (int l = 0; l + 1 < h->L; ++l)
-      if ((s = run_stage(h, l, FS_STAGE_DOWNSAMPLE, 0, st)) != FS_OK) return s;
+    if ((s = enqueue_pyramid(h, I0[i], I1[i], st)) != FS_OK) return s;
   }
   FS_CUDA(cudaMemsetAsync(P->ctrl, 0, P->zero_bytes, st));
   // its items derive the iterations' constants themselves and do not write

@@ -76,6 +76,12 @@ __global__ void k_mask_to_float(const uint8_t* __restrict__ m, float* __restrict
 // (I0 null: I1 only; else also launch_copy_in_image of I0.)
 cudaError_t launch_prerotate(const float* I0, const float* I1, const float4* field,
                              const LevelView& L0, cudaStream_t st);
+// launch_prerotate of both images and launch_downsample down to level n - 1
+// (n <= kPyramidLevels) in one launch, the same values.
+constexpr int kPyramidLevels = 5;
+int pyramid_blocks(const LevelView& L0);   // its grid
+cudaError_t launch_pyramid(const float* I0, const float* I1, const float4* field,
+                           const LevelView* const* levels, int n, cudaStream_t st);
 // A dense FP32 image into level L's I0 (which = 0) or I1 (1), with the low
 // part of its rounding to the level's storage (the pyramid's carry).
 cudaError_t launch_copy_in_image(const float* src, const LevelView& L, int which,
@@ -183,7 +189,9 @@ cudaError_t launch_pd_consts(const LevelView& L, float lam, float eps, cudaStrea
 // for it before reading the state.  PD_CHAIN_START when it directly follows
 // the launch of this library that wrote the constants (launch_warp,
 // launch_clip_warp): a programmatic dependent launch too, which waits before
-// it reads anything.  0: an ordinary launch.
+// it reads anything.  PD_CHAIN_WARP when that was a launch_clip_warp with
+// `keep` in such a chain: all constants but step and c0 are read before the
+// wait.  0: an ordinary launch.
 cudaError_t launch_pd(int variant, const LevelView& L, const PDState& in, const PDState& out,
                       const PDParams& pp, int B, int n, cudaStream_t st, int chained = 0);
 

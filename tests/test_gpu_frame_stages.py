@@ -12,6 +12,28 @@ pytestmark = pytest.mark.gpu
 WARPS, ITERS, LEVELS = 2, 7, 2
 
 
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("W, H, levels", [(203, 157, 6), (17, 40, 3), (64, 41, 2), (15, 16, 1),
+                                          (393, 385, 5), (401, 400, 5)])
+def test_pyramid_equals_its_stages(W, H, levels, storage):
+    # both sides of the size rule, ragged edges, more levels than one launch makes
+    p = f32pair(ragged_pair(4, W=W, H=H))
+    outs = []
+    for stages in (False, True):
+        s = make_solver(p, levels=levels, storage=storage)
+        if stages:
+            s.write(0, "I0", p["I0"])
+            s.prerotate(p["I1"])
+            for l in range(levels - 1):
+                s.stage(l, "DOWNSAMPLE")
+        else:
+            s.solve(p["I0"], p["I1"], 1, 1)
+        outs.append([np64(s.read(l, b)) for l in range(levels) for b in ("I0", "I1")])
+        s.close()
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b)
+
+
 def _warps(s, level):
     s.stage(level, "WARP")
     for w in range(WARPS):
