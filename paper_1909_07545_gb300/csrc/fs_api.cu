@@ -68,8 +68,10 @@ struct HostLevel {
   int tuned = -1;                           // autotuned choice: 0 cluster, 1..8 depth, -1 none
   int tuned_variant = -1;                   // autotuned tile variant, -1: by size
   // pd_auto's last answer and what it was asked (pd_plan)
-  mutable PdSchedule plan;
-  mutable int plan_iters = -1, plan_nl = -1;
+  // ([1]: odd numbers of launches too)
+  mutable PdSchedule plan[2];
+  mutable int plan_iters[2] = {-1, -1}, plan_nl[2] = {-1, -1};
+  bool flipped = false;                     // the two buffer sets have changed places (flip_sets)
   bool auto_best = false;                   // the tuner found pd_auto's schedule faster still
   LevelView v{};
   // tensor maps of the TMA-staged primal-dual footprints, reading buffer
@@ -450,7 +452,7 @@ bool use_cluster(const fs_handle* h, int l) {
 // launches, and so does 16-bit storage (depth 6 on levels wider than 512 px,
 // 8 below), whose results depend on it.  A halo is never deeper than the
 // longest launch's iterations.
-PdSchedule pd_plan(const fs_handle* h, int l, int iters) {
+PdSchedule pd_plan(const fs_handle* h, int l, int iters, bool odd = false) {
   const HostLevel& L = h->lv[l];
   const int b = std::min(h->prm.block_iters, 8);
   const bool tgv = h->prm.regularizer == FS_REG_TGV;
@@ -466,19 +468,22 @@ PdSchedule pd_plan(const fs_handle* h, int l, int iters) {
     nl = pd_launch_count(iters, b > 0 ? b : (L.W > 512 || L.H > 512) ? 6 : 8);
   else if (b > 0 && (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0))
     nl = pd_launch_count(iters, b);
-  if (L.plan_iters != iters || L.plan_nl != nl) {
-    L.plan = tgv ? tgv_auto(L.v, iters, nl, h->sms) : pd_auto(L.v, iters, nl, h->sms, L.tma_ok);
-    L.plan_iters = iters;
-    L.plan_nl = nl;
+  const int k = odd ? 1 : 0;
+  if (L.plan_iters[k] != iters || L.plan_nl[k] != nl) {
+    L.plan[k] = tgv ? tgv_auto(L.v, iters, nl, h->sms)
+                    : pd_auto(L.v, iters, nl, h->sms, L.tma_ok, odd);
+    L.plan_iters[k] = iters;
+    L.plan_nl[k] = nl;
   }
-  return L.plan;
+  return L.plan[k];
 }
 
 // Whether a solve of h with `iters` iterations a warp runs the TMA-staged footprints on some level.
 bool uses_tma(const fs_handle* h, int iters) {
   if (h->prm.regularizer == FS_REG_TGV) return false;
   for (int l = 0; l < h->L; ++l)
-    if (!use_cluster(h, l) && pd_plan(h, l, iters).variant == PD_TILE_64_TMA) return true;
+    for (bool odd : {false, true})
+      if (!use_cluster(h, l) && pd_plan(h, l, iters, odd).variant == PD_TILE_64_TMA) return true;
   return false;
 }
 
@@ -489,10 +494,38 @@ bool uses_tma(const fs_handle* h, int iters) {
 // levels of 128 x 128: 211 -> 170 us.  With 8 launches a warp the chain's
 // reading of the constants through L2 costs more than the gaps, 505 -> 526
 // us on 256 x 256; with 4 it still loses 2 %.)
-bool short_chain(const fs_handle* h, int l, int iters) {
+bool short_chain(const fs_handle* h, int l, int iters, bool odd) {
   return h->prm.regularizer == FS_REG_HUBER_TV && !use_cluster(h, l) &&
-         pd_plan(h, l, iters).launches <= 2;
+         pd_plan(h, l, iters, odd).launches <= 2;
 }
+
+// Whether warp w of `warps` on a level may take an odd number of launches.
+// They leave the state in the level's other buffer set, which then counts as
+// the first one (flip_sets); two such warps bring it back, so the last of an
+// odd number of warps may not.  (50 iterations a warp on 256 x 256, 3 levels:
+// 484.8 -> 440.1 us a frame; 10 on 800 x 800, 5 levels: 1597 -> 1560.)
+bool odd_launches(const fs_handle* h, int w, int warps) {
+  return h->prm.regularizer == FS_REG_HUBER_TV && w < warps / 2 * 2;
+}
+
+void flip_sets(HostLevel& L) {
+  std::swap(L.v.u, L.v.u_alt);
+  std::swap(L.v.ubar, L.v.ubar_alt);
+  std::swap(L.v.p1, L.v.p1_alt);
+  std::swap(L.v.p2, L.v.p2_alt);
+  std::swap(L.tma[0], L.tma[1]);
+  L.flipped = !L.flipped;
+}
+
+// Puts the sets back where work being enqueued stops with an error.
+struct SetsGuard {
+  fs_handle* h;
+  ~SetsGuard() {
+    for (int l = 0; l < h->L; ++l)
+      if (h->lv[l].flipped) flip_sets(h->lv[l]);
+  }
+};
+
 
 // The accelerated schedule's table for at least `iters` iterations per
 // warp, built in FP64 on the host and stored as FP32 (synchronous; called
@@ -533,9 +566,11 @@ fs_status ensure_schedule(fs_handle* h, int iters) {
 }
 
 // chain: the launch before on the stream is this library's warp start of the
-// level (the first launch may then be a programmatic dependent one).
+// level, the first (warp = 0) or a later one (the first launch may then be a
+// programmatic dependent one).  odd: an odd number of launches may change
+// the sets' places.
 fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = false,
-                 int warp = 0) {
+                 int warp = 0, bool odd = false) {
   HostLevel& L = h->lv[l];
   PDParams pp{h->prm.lambda, h->prm.huber_eps, h->prm.theta};
   if (h->prm.accel_gamma > 0) {
@@ -558,13 +593,13 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
       return fail(FS_ECUDA, "launch of k_pd_cluster failed: %s", cudaGetErrorString(e));
     return FS_OK;
   }
-  const PdSchedule ps = pd_plan(h, l, iters);
+  const PdSchedule ps = pd_plan(h, l, iters, odd);
   const int variant = ps.variant, B = ps.depth, nl = ps.launches;
   PDState A{L.v.u, L.v.ubar, L.v.p1, L.v.p2};
   PDState Bs{L.v.u_alt, L.v.ubar_alt, L.v.p1_alt, L.v.p2_alt};
   const bool tma = variant == PD_TILE_64_TMA;
   if (tma && !L.tma_ok) return fail(FS_EINVAL, "level %d: no tensor maps for the TMA footprints", l);
-  pp.fresh = chain && !L.consts_stale && short_chain(h, l, iters);
+  pp.fresh = chain && !L.consts_stale && short_chain(h, l, iters, odd);
   if (L.consts_stale) {
     FS_LAUNCH("k_pd_consts", launch_pd_consts(L.v, h->prm.lambda, h->prm.huber_eps, st));
     L.consts_stale = false;
@@ -589,7 +624,9 @@ fs_status run_pd(fs_handle* h, int l, int iters, cudaStream_t st, bool chain = f
                   cudaGetErrorString(e));
     done += n;
   }
-  if (nl % 2 == 1) {   // a single launch: bring the state back to the primary set
+  if (nl % 2 == 1 && odd) {
+    flip_sets(L);
+  } else if (nl % 2 == 1) {   // a single launch: bring the state back to the primary set
     size_t bytes = (size_t)L.P * L.H * sizeof(float);
     size_t sbytes = (size_t)L.P * L.H * storage_size(L.v.st);
     FS_CUDA(cudaMemcpyAsync(A.u, Bs.u, bytes, cudaMemcpyDeviceToDevice, st));
@@ -709,9 +746,9 @@ fs_status enqueue_depth(fs_handle* h, float* disp, float* depth, cudaStream_t st
 // The end of a warp (clip + update, Eq. 8-9) in one launch with what follows:
 // the next warp's start (warp + linearise), or after a frame's last warp the
 // triangulation.
-fs_status end_warp(fs_handle* h, int l, int iters, bool next, float* disp, float* depth,
+fs_status end_warp(fs_handle* h, int l, int iters, bool odd, bool next, float* disp, float* depth,
                    cudaStream_t st) {
-  const bool chain = short_chain(h, l, iters);
+  const bool chain = short_chain(h, l, iters, odd);
   if (next || l > 0) return run_stage(h, l, next ? FS_STAGE_CLIP_WARP : FS_STAGE_CLIP, 0, st, chain);
   HostLevel& L0 = h->lv[0];
   L0.consts_stale = true;
@@ -742,6 +779,7 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
                         cudaEvent_t finest_wait = nullptr, cudaEvent_t finest_done = nullptr,
                         bool cont = false) {
   NvtxRange range(init || cont ? "fs warm solve" : "fs solve");
+  SetsGuard guard{h};
   fs_status s;
   HostLevel& L0 = h->lv[0];
   int top = h->L - 1;
@@ -757,10 +795,11 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
       if ((s = start_level(h, 0, START_GIVEN, st)) != FS_OK) return s;
     }
     for (int w = 0; w < warps; ++w) {
+      const bool odd = odd_launches(h, w, warps);
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w], st));
-      if ((s = run_pd(h, 0, iters, st, true, w)) != FS_OK) return s;
+      if ((s = run_pd(h, 0, iters, st, true, w, odd)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * w + 1], st));
-      if ((s = end_warp(h, 0, iters, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
+      if ((s = end_warp(h, 0, iters, odd, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
     }
     if (h->timing) {
       h->ev_warps = warps;
@@ -781,10 +820,11 @@ fs_status enqueue_solve(fs_handle* h, const float* I0, const float* I1, const fl
     if (l == 0 && finest_wait) FS_CUDA(cudaStreamWaitEvent(st, finest_wait, 0));
     if ((s = start_level(h, l, l == top ? START_ZERO : START_UPSAMPLE, st)) != FS_OK) return s;
     for (int w = 0; w < warps; ++w) {
+      const bool odd = odd_launches(h, w, warps);
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w)], st));
-      if ((s = run_pd(h, l, iters, st, true, w)) != FS_OK) return s;
+      if ((s = run_pd(h, l, iters, st, true, w, odd)) != FS_OK) return s;
       if (h->timing) FS_CUDA(record_event(h->ev[2 * (l * warps + w) + 1], st));
-      if ((s = end_warp(h, l, iters, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
+      if ((s = end_warp(h, l, iters, odd, w + 1 < warps, disp, depth, st)) != FS_OK) return s;
     }
   }
   if (h->timing) {
@@ -2005,9 +2045,10 @@ extern "C" fs_status fs_timing_read(fs_handle* h, double* ms, long long* launche
                                      h->ev[2 * (l * h->ev_warps + w) + 1]));
         h->t_ms[l] += t;
       }
-      h->t_launch[l] += use_cluster(h, l)
-                            ? (long long)h->ev_warps
-                            : (long long)h->ev_warps * pd_plan(h, l, h->ev_iters).launches;
+      for (int w = 0; w < h->ev_warps; ++w)
+        h->t_launch[l] += use_cluster(h, l) ? 1
+                                            : pd_plan(h, l, h->ev_iters,
+                                                      odd_launches(h, w, h->ev_warps)).launches;
       h->t_pxit[l] += (double)h->lv[l].W * h->lv[l].H * h->ev_warps * h->ev_iters;
     }
     h->ev_pending = false;

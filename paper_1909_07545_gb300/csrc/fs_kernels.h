@@ -115,9 +115,10 @@ struct BlockFit {
 };
 // The least of the modelled times over n_fit footprints and launch counts.
 PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, int iters,
-                          int launches, int sms);
-// Huber-TV; tma: the TMA-staged footprints may be chosen
-PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma);
+                          int launches, int sms, bool odd = false);
+// Huber-TV; tma: the TMA-staged footprints may be chosen; odd: an odd number
+// of launches too
+PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma, bool odd);
 PdSchedule tgv_auto(const LevelView& L, int iters, int launches, int sms);   // TGV-L1
 // Launches of `iters` iterations at most `depth` each, made even when
 // iters >= 2 so that the ping-pong state ends where it began.

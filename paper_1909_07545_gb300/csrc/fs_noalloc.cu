@@ -176,7 +176,8 @@ extern "C" fs_status fs_pd_iterate_noalloc(const float* d_I0, const unsigned cha
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const PdSchedule ps =
-      pd_auto(L, iters, p.block_iters > 0 ? pd_launch_count(iters, p.block_iters) : 0, sms, false);
+      pd_auto(L, iters, p.block_iters > 0 ? pd_launch_count(iters, p.block_iters) : 0, sms, false,
+              false);
   const int nl = ps.launches;
   PDParams pp{p.lambda, p.huber_eps, p.theta};
   PDState A{L.u, L.ubar, L.p1, L.p2};

@@ -272,7 +272,8 @@ int pd_launch_count(int iters, int depth) {
 // Where it saves waves, the footprints outside the FOV are left out: a 2048 x
 // 2048 frame under a 180-degree lens takes 24.0 ms against 27.9.  (With a
 // single wave the test only costs, up to 4 % of a 256 x 256 frame.)
-PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma) {
+PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma,
+                   bool odd) {
   static const BlockFit kFit[] = {
       {PD_TILE_32x16_T256, 32, 16, 1, 1.95f, 0.18f, false},
       {PD_TILE_32x24_T384, 32, 24, 1, 1.85f, 0.185f, false},
@@ -287,7 +288,7 @@ PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tm
       {PD_TILE_64_TMA, 64, 64, 1, 2.3f, 0.78f, true, 48, 2.8f},
   };
   return block_schedule(kFit, (int)(sizeof(kFit) / sizeof(kFit[0])) - !tma, L, iters, launches,
-                        sms);
+                        sms, odd);
 }
 
 void fov_columns(const LevelView& L, int pitch, int x0, int fw, int fh, int tiles_x, int y0,
@@ -305,7 +306,7 @@ void fov_columns(const LevelView& L, int pitch, int x0, int fw, int fh, int tile
 }
 
 PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, int iters,
-                          int launches, int sms) {
+                          int launches, int sms, bool odd) {
   constexpr int kMaxDepth = 15;
   PdSchedule best;
   best.launches = launches > 0 ? launches : pd_launch_count(iters, 8);
@@ -322,7 +323,7 @@ PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, in
       const double seats = (double)f.per_sm * sms;
       double waves = std::ceil((double)tx * ty / seats);
       bool skip = false;
-      if (f.skip && waves > 1.0 && nl > 1) {
+      if (f.skip && waves > 1.0 && nl % 2 == 0) {   // (pd_idle works in place)
         double active = 0;           // footprints that may hold FOV pixels
         for (int y = 0; y < ty; ++y) {
           int lo, hi;
@@ -345,7 +346,10 @@ PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, in
   } else if (iters < 2) {
     consider(1);
   } else {
-    for (int depth = kMaxDepth; depth >= 3; --depth) consider(pd_launch_count(iters, depth));
+    for (int depth = kMaxDepth; depth >= 3; --depth) {
+      consider(pd_launch_count(iters, depth));
+      if (odd) consider((iters + depth - 1) / depth);
+    }
   }
   if (best.depth == 0) best.depth = std::max(1, (iters + best.launches - 1) / best.launches);
   return best;

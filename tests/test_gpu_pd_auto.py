@@ -101,6 +101,28 @@ def test_large_levels_and_footprints_outside_the_fov(W, H, iters, prm):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("prm", [dict(), dict(precond=0, accel_gamma=0.3), dict(storage="f16")])
+@pytest.mark.parametrize("warps, iters", [(1, 10), (2, 1), (3, 10), (4, 25), (5, 1)])
+def test_odd_launch_counts(warps, iters, prm):
+    # an odd number of launches leaves the state in the other buffer set: after
+    # a frame of any number of warps, and one continued from it, all state is
+    # where the explicit schedules (even counts, copies) leave it
+    p = f32pair(synth.plain_small(1, W=133, H=70, supersample=1))
+    outs = []
+    for choice in (-1, 32):                           # 32: depth 8 on 64 x 64
+        s = make_solver(p, levels=2, pd_schedule=1, **prm)
+        s.set_schedule([choice, choice])
+        s.timing_enable(True)
+        out = list(s.solve(p["I0"], p["I1"], warps, iters))
+        out += s.solve_continue(p["I1"], p["I0"], warps, iters)
+        out += [s.read(l, b) for l in (0, 1) for b in ("U", "UBAR", "UW", "P", "W")]
+        s.timing_read()
+        outs.append([np64(x) for x in out])
+        s.close()
+    for a, b in zip(*outs):
+        assert np.array_equal(a, b, equal_nan=True)
+
+
 TGV = ("U", "UBAR", "V", "VBAR", "P", "Q")
 
 
