@@ -332,8 +332,8 @@ __global__ void k_warm_start(LevelView L, float du_max) {
 // disparities count as 0 (with w = 0).
 template <int S>
 __device__ __forceinline__ float continue_px(const LevelView& L, size_t i, bool in, float2& w) {
-  float d = L.u[i];
-  w = L.w[i];
+  float d = ldf<true>(L.u + i);
+  w = ldf2<true>(L.w + i);
   if (!in || !isfinite(d)) {
     d = 0.f;
     w = make_float2(0.f, 0.f);
@@ -441,11 +441,15 @@ __global__ void k_warp(LevelView L, int central, float lam, float eps, int const
 // k_zero_state, k_upsample, k_continue or nothing, then k_warp, whose results
 // a pixel only needs of itself.  A level started with three to five launches,
 // each of a few microseconds on the small levels: a 128 x 128 frame of 3
-// levels, all in all, went from 169 to 141 us, an 800 x 800 frame of 3 from 1707
-// to 1684.
+// levels, all in all, went from 169 to 141 us, an 800 x 800 frame of 5 from 1707
+// to 1684.  A programmatic dependent launch that waits first, which starts
+// sooner than an ordinary one; so what the launch before wrote besides images
+// is read through L2.  128 x 128:
+// 126.4 -> 120.8.
 template <int S, int MODE, bool TGV>
 __global__ void k_level_start(LevelView C, LevelView L, float beta, float eta, int precond,
                               int central, float lam, float eps, int consts) {
+  cudaGridDependencySynchronize();
   int x = blockIdx.x * blockDim.x + threadIdx.x;
   int y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= L.W || y >= L.H) return;
@@ -457,12 +461,12 @@ __global__ void k_level_start(LevelView C, LevelView L, float beta, float eta, i
   if constexpr (MODE == START_ZERO) {
     zero_px<S>(L, i);
   } else if constexpr (MODE == START_UPSAMPLE) {
-    u = upsample_px<S, false>(C, L, x, y, w);
+    u = upsample_px<S, true>(C, L, x, y, w);
   } else if constexpr (MODE == START_CONTINUE) {
     u = continue_px<S>(L, i, in, w);
   } else {
-    u = L.u[i];
-    w = L.w[i];
+    u = ldf<true>(L.u + i);
+    w = ldf2<true>(L.w + i);
   }
   if constexpr (TGV && MODE != START_GIVEN) {
     L.v1[i] = L.v2[i] = 0.f;
@@ -772,9 +776,9 @@ cudaError_t launch_level_start(int mode, const LevelView& C, const LevelView& L,
                                float eta, int precond, int central, float lam, float eps,
                                int consts, cudaStream_t st) {
   if (consts != WARP_CONSTS_HUBER)
-    return launch_chained(level_start_kernel<ST_F32, true>(mode), L, false, st, C, L, beta, eta,
+    return launch_chained(level_start_kernel<ST_F32, true>(mode), L, true, st, C, L, beta, eta,
                           precond, central, lam, eps, consts);
-  FS_STORAGE_SWITCH(L.st, return launch_chained(level_start_kernel<S, false>(mode), L, false, st,
+  FS_STORAGE_SWITCH(L.st, return launch_chained(level_start_kernel<S, false>(mode), L, true, st,
                                                 C, L, beta, eta, precond, central, lam, eps,
                                                 consts))
 }
