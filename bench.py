@@ -938,7 +938,7 @@ def main():
                    "l2": "flushed between steps (256 MB write)",
                    "pd_schedule_per_level": (
                        [schedule_label(c) for c in tuned]
-                       if tuned else "default (cluster <= 128 px, blocking 6 / 8 above)"),
+                       if tuned else "default (footprint and depth by level size and iterations)"),
                    "autotuned": bool(tuned), "graph": True,
                    "parallelism": f"replicas x{world}"},
         "latency_ms": {"p50": float(np.percentile(step_ms, 50)),

@@ -1,8 +1,7 @@
 // df.cuh -- float-float arithmetic for the kernels whose FP32 rounding the
 // warping would amplify: the trajectory field, the calibration field, the
 // pre-rotation and the image pyramid.  They run once per pose or once per
-// frame, so their cost does not matter; what matters is that each stored
-// result is its exact value rounded once to float.
+// frame; each stored result is its exact value rounded once to float.
 //
 // A value is the unevaluated sum hi + lo of two floats with |lo| <= ulp(hi)/2
 // (about 48 significant bits).  Every step is FP32 arithmetic:

@@ -121,7 +121,7 @@ PdSchedule block_schedule(const BlockFit* fit, int n_fit, const LevelView& L, in
 PdSchedule pd_auto(const LevelView& L, int iters, int launches, int sms, bool tma, bool odd);
 PdSchedule tgv_auto(const LevelView& L, int iters, int launches, int sms);   // TGV-L1
 // Launches of `iters` iterations at most `depth` each, made even when
-// iters >= 2 so that the ping-pong state ends where it began.
+// iters >= 2 so that the state ends in the buffer set it began in.
 int pd_launch_count(int iters, int depth);
 
 // TGV-L1 (k_tgv.cu): n iterations, with ps.launches = 0 as a dual and a

@@ -168,8 +168,8 @@ extern "C" fs_status fs_pd_iterate_noalloc(const float* d_I0, const unsigned cha
     return fs_internal_set_error(FS_ECUDA, msg);
   }
 
-  // same launch schedule as the handle path: an even number of launches, so
-  // the state ends in the caller's buffers, each but the first chained to
+  // the handle path's schedule with an even number of launches, so the state
+  // ends in the caller's buffers, each but the first chained to
   // the one before (the constants were written before the first)
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);

@@ -437,15 +437,13 @@ __global__ void k_warp(LevelView L, int central, float lam, float eps, int const
 }
 
 // The start of a level in one pass: tensor and step sizes, the start state
-// (MODE), and the first warp's linearisation and constants -- k_tensor, then
-// k_zero_state, k_upsample, k_continue or nothing, then k_warp, whose results
-// a pixel only needs of itself.  A level started with three to five launches,
+// (MODE), and the first warp's linearisation and constants: k_tensor, the
+// start state and k_warp, whose results a pixel only needs of itself.  A level started with three to five launches,
 // each of a few microseconds on the small levels: a 128 x 128 frame of 3
 // levels, all in all, went from 169 to 141 us, an 800 x 800 frame of 5 from 1707
 // to 1684.  A programmatic dependent launch that waits first, which starts
 // sooner than an ordinary one; so what the launch before wrote besides images
-// is read through L2.  128 x 128:
-// 126.4 -> 120.8.
+// is read through L2: 128 x 128 126.4 -> 120.8 us.
 template <int S, int MODE, bool TGV>
 __global__ void k_level_start(LevelView C, LevelView L, float beta, float eta, int precond,
                               int central, float lam, float eps, int consts) {

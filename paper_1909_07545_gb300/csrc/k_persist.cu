@@ -99,7 +99,7 @@ __device__ __forceinline__ void for_tile_pixels(const PersistJob& J, int bx, int
 }
 
 // PRE: what the stage kernels TENSOR, zero state or UPSAMPLE, then WARP do at
-// these pixels (k_tensor, k_zero_state / k_upsample, k_warp).
+// these pixels (k_level_start).
 template <int S>
 __device__ __noinline__ void pre_item(const PersistJob& J, int bx, int by) {
   const LevelView& L = J.L;

@@ -9,8 +9,8 @@
 //     state in place (each pixel reads its right / lower neighbours in the
 //     dual and its left / upper ones in the primal, so the launch boundary is
 //     the only synchronisation needed);
-//   * temporal blocking (k_tgv_blocked): a CTA keeps a 32 x 32 footprint's
-//     whole state (u, ubar, v, vbar, p, q: 12 values per pixel) in registers
+//   * temporal blocking (k_tgv_blocked): a CTA keeps a footprint's (32 x 16
+//     to 64 x 32 pixels; tgv_auto or the tuner picks one per level) whole state (u, ubar, v, vbar, p, q: 12 values per pixel) in registers
 //     for n <= B iterations, exchanging ubar, vbar and the masked products
 //     T^1/2 p and q with its neighbours through shared memory; the outer B
 //     pixels of the footprint are halo, recomputed by the neighbouring CTAs.
