@@ -110,12 +110,14 @@ __device__ __forceinline__ TensorAt tensor_at(const LevelView& L, int x, int y, 
 //   sigma(x) = 1 / max(2(|a| m1 + |b| m2), 2(|b| m1 + |c| m2))
 //   tau(x)   = 1 / ((|a|+|b|) m1 + (|b|+|c|) m2 at x,
 //                   + (|a|+|b|) m1 at x - e1, + (|b|+|c|) m2 at x - e2)
-template <int S>
-__device__ __forceinline__ void tensor_px(const LevelView& L, int x, int y, float beta, float eta,
-                                          int precond) {
+// left(), up(): |a| + |b| at x - e1 and |b| + |c| at x - e2 (called where the
+// difference there is active).
+template <int S, class Left, class Up>
+__device__ __forceinline__ void tensor_store_px(const LevelView& L, int x, int y,
+                                                const TensorAt& t, int precond, Left left,
+                                                Up up) {
   size_t i = (size_t)y * L.P + x;
   uint8_t m = L.mask[i];
-  TensorAt t = tensor_at<S>(L, x, y, beta, eta);
   sst<S>(L.sx, i, t.sx);
   sst<S>(L.sy, i, t.sy);
   if (!precond) {
@@ -130,15 +132,24 @@ __device__ __forceinline__ void tensor_px(const LevelView& L, int x, int y, floa
   float r = fmaxf(r1, r2);
   L.sig[i] = r > 0.f ? 1.f / r : 0.f;
   float col = (t.aa + t.bb) * m1 + (t.bb + t.cc) * m2;
-  if (x > 0 && (L.mask[i - 1] & MASK_GX)) {
-    TensorAt tl = tensor_at<S>(L, x - 1, y, beta, eta);
-    col += tl.aa + tl.bb;
-  }
-  if (y > 0 && (L.mask[i - L.P] & MASK_GY)) {
-    TensorAt tu = tensor_at<S>(L, x, y - 1, beta, eta);
-    col += tu.bb + tu.cc;
-  }
+  if (x > 0 && (L.mask[i - 1] & MASK_GX)) col += left();
+  if (y > 0 && (L.mask[i - L.P] & MASK_GY)) col += up();
   L.tau[i] = (col > 0.f && (m & MASK_IN)) ? 1.f / col : 0.f;
+}
+
+template <int S>
+__device__ __forceinline__ void tensor_px(const LevelView& L, int x, int y, float beta, float eta,
+                                          int precond) {
+  tensor_store_px<S>(
+      L, x, y, tensor_at<S>(L, x, y, beta, eta), precond,
+      [&] {
+        const TensorAt t = tensor_at<S>(L, x - 1, y, beta, eta);
+        return t.aa + t.bb;
+      },
+      [&] {
+        const TensorAt t = tensor_at<S>(L, x, y - 1, beta, eta);
+        return t.bb + t.cc;
+      });
 }
 
 
