@@ -168,7 +168,7 @@ fs_status fs_set_wait_limit(fs_handle* h, double seconds);
 /* Testing aid for the bound above: stall = 1 makes the first work items of
  * the finest level of this handle's persistent solves wait for a counter
  * that nothing advances, so that wait runs out, and makes the first launch
- * of every level that runs the TMA-staged footprints (choices 56..63) wait
+ * of every level that runs the TMA-staged footprints (below) wait
  * for 16 bytes that no copy delivers; stall = 0 restores the schedule.  A
  * batch stalls when any of its handles does.  Both this call and
  * fs_set_wait_limit drop the handle's captured graph (the bound and the
@@ -176,8 +176,8 @@ fs_status fs_set_wait_limit(fs_handle* h, double seconds);
  * captured with. */
 fs_status fs_persist_stall(fs_handle* h, int stall);
 
-/* The TMA-staged primal-dual footprints (fs_autotune choices 56..63): each
- * launch's CTAs wait on a shared-memory barrier for the copies of every
+/* The TMA-staged primal-dual footprints (fs_autotune choices 56..63, and the
+ * automatic schedule's choice on the largest levels): each launch's CTAs wait on a shared-memory barrier for the copies of every
  * footprint, bounded like the persistent schedule (fs_set_wait_limit).  A
  * wait that runs out makes its CTA return and records FS_ETIMEOUT in the
  * handle.  fs_check_waits synchronises the handle's stream and returns
