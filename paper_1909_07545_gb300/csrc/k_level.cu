@@ -481,7 +481,8 @@ __global__ void k_level_start(LevelView C, LevelView L, float beta, float eta, i
   size_t i = (size_t)y * L.P + x;
   const bool in = L.mask[i] & MASK_IN;
   tensor_store_px<S>(
-      L, x, y, t, precond, [&] { return s_h[ty][tx]; }, [&] { return s_v[ty][tx]; });
+      L, x, y, t, precond, L.mask[i], x > 0 && (L.mask[i - 1] & MASK_GX),
+      y > 0 && (L.mask[i - L.P] & MASK_GY), [&] { return s_h[ty][tx]; }, [&] { return s_v[ty][tx]; });
   float u = 0.f;
   float2 w = make_float2(0.f, 0.f);
   if constexpr (MODE == START_ZERO) {

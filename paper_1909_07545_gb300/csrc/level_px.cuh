@@ -73,18 +73,19 @@ struct TensorAt {
 // T^1/2 = e n n^T + n_perp n_perp^T = I - (1 - e) n n^T  (Eq. 12) with
 // e = exp(-beta |grad I0|^eta), grad I0 by central differences on the mask
 // (one-sided at its edge, 0 where both neighbours leave it).
-template <int S>
-__device__ __forceinline__ TensorAt tensor_at(const LevelView& L, int x, int y, float beta,
-                                              float eta) {
+// in(i): whether pixel i is inside the mask.
+template <int S, class In>
+__device__ __forceinline__ TensorAt tensor_in(const LevelView& L, int x, int y, float beta,
+                                              float eta, In in) {
   TensorAt t;
   size_t i = (size_t)y * L.P + x;
-  if (!(L.mask[i] & MASK_IN)) { t.sx = t.sy = 0.f; t.aa = 1.f; t.bb = 0.f; t.cc = 1.f; return t; }
+  if (!in(i)) { t.sx = t.sy = 0.f; t.aa = 1.f; t.bb = 0.f; t.cc = 1.f; return t; }
   auto I0 = [&](size_t k) { return sld<S>(L.I0, k); };
   float c = I0(i);
-  bool r = x + 1 < L.W && (L.mask[i + 1] & MASK_IN);
-  bool l = x > 0 && (L.mask[i - 1] & MASK_IN);
-  bool d = y + 1 < L.H && (L.mask[i + L.P] & MASK_IN);
-  bool u = y > 0 && (L.mask[i - L.P] & MASK_IN);
+  bool r = x + 1 < L.W && in(i + 1);
+  bool l = x > 0 && in(i - 1);
+  bool d = y + 1 < L.H && in(i + L.P);
+  bool u = y > 0 && in(i - L.P);
   float gx = 0.f, gy = 0.f;
   if (r && l) gx = 0.5f * (I0(i + 1) - I0(i - 1));
   else if (r) gx = I0(i + 1) - c;
@@ -105,19 +106,24 @@ __device__ __forceinline__ TensorAt tensor_at(const LevelView& L, int x, int y, 
   return t;
 }
 
+template <int S>
+__device__ __forceinline__ TensorAt tensor_at(const LevelView& L, int x, int y, float beta,
+                                              float eta) {
+  return tensor_in<S>(L, x, y, beta, eta, [&](size_t i) { return (L.mask[i] & MASK_IN) != 0; });
+}
+
 // Diagonal preconditioning (Pock-Chambolle 2011, alpha = 1) from the row and
 // column sums of the entrywise bound |T^1/2| |grad| of K = T^1/2 grad:
 //   sigma(x) = 1 / max(2(|a| m1 + |b| m2), 2(|b| m1 + |c| m2))
 //   tau(x)   = 1 / ((|a|+|b|) m1 + (|b|+|c|) m2 at x,
 //                   + (|a|+|b|) m1 at x - e1, + (|b|+|c|) m2 at x - e2)
-// left(), up(): |a| + |b| at x - e1 and |b| + |c| at x - e2 (called where the
-// difference there is active).
+// m: the pixel's mask bits; gx_left, gy_up: whether the differences at x - e1
+// and x - e2 are active; left(), up(): |a| + |b| and |b| + |c| there.
 template <int S, class Left, class Up>
 __device__ __forceinline__ void tensor_store_px(const LevelView& L, int x, int y,
-                                                const TensorAt& t, int precond, Left left,
-                                                Up up) {
+                                                const TensorAt& t, int precond, unsigned m,
+                                                bool gx_left, bool gy_up, Left left, Up up) {
   size_t i = (size_t)y * L.P + x;
-  uint8_t m = L.mask[i];
   sst<S>(L.sx, i, t.sx);
   sst<S>(L.sy, i, t.sy);
   if (!precond) {
@@ -132,16 +138,18 @@ __device__ __forceinline__ void tensor_store_px(const LevelView& L, int x, int y
   float r = fmaxf(r1, r2);
   L.sig[i] = r > 0.f ? 1.f / r : 0.f;
   float col = (t.aa + t.bb) * m1 + (t.bb + t.cc) * m2;
-  if (x > 0 && (L.mask[i - 1] & MASK_GX)) col += left();
-  if (y > 0 && (L.mask[i - L.P] & MASK_GY)) col += up();
+  if (gx_left) col += left();
+  if (gy_up) col += up();
   L.tau[i] = (col > 0.f && (m & MASK_IN)) ? 1.f / col : 0.f;
 }
 
 template <int S>
 __device__ __forceinline__ void tensor_px(const LevelView& L, int x, int y, float beta, float eta,
                                           int precond) {
+  const size_t i = (size_t)y * L.P + x;
   tensor_store_px<S>(
-      L, x, y, tensor_at<S>(L, x, y, beta, eta), precond,
+      L, x, y, tensor_at<S>(L, x, y, beta, eta), precond, L.mask[i],
+      x > 0 && (L.mask[i - 1] & MASK_GX), y > 0 && (L.mask[i - L.P] & MASK_GY),
       [&] {
         const TensorAt t = tensor_at<S>(L, x - 1, y, beta, eta);
         return t.aa + t.bb;
