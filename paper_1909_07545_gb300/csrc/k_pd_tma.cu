@@ -29,7 +29,8 @@
 // The planes of the next footprint are requested only after the CTA barrier
 // that follows every thread's reads of the current one.  Every wait is
 // bounded by wait_ns of global time; a wait that runs out sets *status to
-// FS_ETIMEOUT and the CTA returns.
+// FS_ETIMEOUT and the CTA returns, one thread of it only once the copies it
+// has under way have landed (or two seconds later).
 #include <algorithm>
 
 #include "fs.h"
@@ -43,6 +44,7 @@ namespace {
 constexpr int kFW = 64, kNY = 16, kR = 4, kFH = kNY * kR;   // 64 x 64, 1024 threads
 constexpr int kIW = 48, kXM = 8;                             // interior columns, column margin
 constexpr int kMaskW = 80, kMaskOff = 16;                    // mask box: 80 columns from 48 bx - 16
+constexpr unsigned long long kDrainNs = 2000000000ull;       // a CTA's last wait for its own copies
 
 // Offsets (bytes) of the staged planes, the exchange planes of pd_iterate
 // and the mbarrier in dynamic shared memory; all multiples of 128.
@@ -141,7 +143,7 @@ __device__ __forceinline__ float sval(const unsigned char* plane, int k) {
 // set `in` and written to `out`.  chained (pd_tile): PD_CHAINED requests the
 // first footprint's constants before the wait for the preceding launch and
 // its state after, PD_CHAIN_START waits first.  stall: testing aid, the
-// first wait never completes.
+// first wait is on a barrier that nothing completes.
 //
 // Bound by the iterations, 1450-1700 clock cycles each, and by what lies
 // between two footprints: 3800 cycles, the 1400 shared-memory wavefronts of
@@ -168,6 +170,7 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   float(*s_t1)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_t1);
   float(*s_t2)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_t2);
   const uint32_t bar = smem_addr(smem + Lay::bar);
+  const uint32_t wait_bar = smem_addr(smem + Lay::bar + (stall ? 32 : 0));
   volatile int* s_late = reinterpret_cast<volatile int*>(smem + Lay::bar + 16);
 
   // footprint t's place; by: a row at or before it (only ever moves down)
@@ -188,8 +191,9 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   int tile = blockIdx.x, by = 0, bx = tile < ntiles ? column(tile, by) : 0;
   if (leader) {
     mbar_init(bar, 1);
+    if (stall) mbar_init(wait_bar, 1);
     *s_late = 0;
-    if (tile < ntiles) mbar_expect_tx(bar, Lay::tx + (stall ? 16u : 0u));
+    if (tile < ntiles) mbar_expect_tx(bar, Lay::tx);
   }
   __syncthreads();
   if (copy >= 0 && tile < ntiles && !is_state(copy))
@@ -201,7 +205,7 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   unsigned parity = 0;
   while (tile < ntiles) {
     const unsigned long long t0 = global_ns();
-    while (!mbar_try_wait(bar, parity)) {
+    while (!mbar_try_wait(wait_bar, parity)) {
       if (global_ns() - t0 > wait_ns) {
         *s_late = 1;
         break;
@@ -242,7 +246,15 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
     // (s_ub: the last footprint's iterations ended with a barrier.)
     const bool full = __syncthreads_and(mb == 07777u);
     if (*s_late) {
-      if (leader) atomicCAS(status, 0, (int)FS_ETIMEOUT);
+      // the footprint's copies may still be under way (the limit can be as
+      // short as a caller likes), and the shared memory they write is another
+      // CTA's once this one has left: one thread stays for them
+      if (leader) {
+        atomicCAS(status, 0, (int)FS_ETIMEOUT);
+        const unsigned long long t1 = global_ns();
+        while (!mbar_try_wait(bar, parity ^ 1u) && global_ns() - t1 <= kDrainNs) {
+        }
+      }
       return;
     }
     if (n_iters == 0) __syncthreads();   // s_late and s_ub as if iterations followed
