@@ -32,6 +32,7 @@
 // FS_ETIMEOUT and the CTA returns, one thread of it only once the copies it
 // has under way have landed (or two seconds later).
 #include <algorithm>
+#include <atomic>
 
 #include "fs.h"
 #include "fs_kernels.h"
@@ -313,18 +314,21 @@ cudaError_t launch_tma_t(const LevelView& L, const PDState& in, const PDState& o
                          const PDParams& pp, int B, int n, int chained, const PdTmaMaps& maps,
                          int* status, unsigned long long wait_ns, int stall, cudaStream_t st) {
   using Lay = TmaLayout<S>;
-  static bool configured = false;
-  static int sms = 0;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_pd_tma<S, ACC>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Lay::bytes);
+  // the SMs of each device the kernel's shared memory is opted in on (0: not
+  // yet): handles of any device and thread come here
+  constexpr int kDevices = 64;
+  static std::atomic<int> sms_of[kDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int sms = dev < kDevices ? sms_of[dev].load() : 0;
+  if (sms == 0) {
+    e = cudaFuncSetAttribute(k_pd_tma<S, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)Lay::bytes);
     if (e != cudaSuccess) return e;
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
       return e;
-    configured = true;
+    if (dev < kDevices) sms_of[dev].store(sms);
   }
   const int IH = kFH - 2 * B;
   const int tiles_x = (L.W + kIW - 1) / kIW, tiles_y = (L.H + IH - 1) / IH;
