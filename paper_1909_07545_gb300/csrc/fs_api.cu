@@ -847,6 +847,14 @@ fs_status prepare_timing(fs_handle* h, int warps) {
   return FS_OK;
 }
 
+// A solve's launches, replayed graphs included, rewrite sigma, I_u, rho0 and
+// u_w of the levels and leave the constants planes as their last warp start
+// did, or (the persistent schedule) untouched.  The host code that notes this
+// beside each launch runs only while launches are enqueued or captured.
+void constants_stale(fs_handle* h) {
+  for (int l = 0; l < h->L; ++l) h->lv[l].consts_stale = true;
+}
+
 fs_status check_handle(const fs_handle* h) {
   if (!h) return fail(FS_EINVAL, "null handle");
   return FS_OK;
@@ -1084,10 +1092,9 @@ static fs_status enqueue_persist(PersistPlan* P, const std::vector<fs_handle*>& 
     if ((s = enqueue_pyramid(h, I0[i], I1[i], st)) != FS_OK) return s;
   }
   FS_CUDA(cudaMemsetAsync(P->ctrl, 0, P->zero_bytes, st));
-  // its items derive the iterations' constants themselves and do not write
-  // the constant planes
-  for (fs_handle* h : hs)
-    for (int l = 0; l < h->L; ++l) h->lv[l].consts_stale = true;
+  // (its items derive the iterations' constants themselves and do not write
+  // the constant planes)
+  for (fs_handle* h : hs) constants_stale(h);
   FS_LAUNCH("k_persist", launch_persist(P->storage, P->jobs, P->phases, P->items, P->n_items,
                                         P->ctrl, P->done, P->level_done, P->wait_ns, P->grid,
                                         st));
@@ -1461,6 +1468,7 @@ static fs_status solve_persist(fs_handle* h, const float* d_I0, const float* d_I
       h->gwarps = warps;
       h->giters = iters;
     }
+    constants_stale(h);
     FS_CUDA(cudaGraphLaunch(h->gexec, h->stream));
   }
   if (s != FS_OK) return s;
@@ -1515,6 +1523,7 @@ static fs_status solve_launch(fs_handle* h, const float* d_I0, const float* d_I1
     h->giters = iters;
   }
   h->has_state = false;
+  constants_stale(h);
   FS_CUDA(cudaGraphLaunch(h->gexec, h->stream));
   h->has_state = true;
   if (h->timing) {              // the replay re-records the captured events
@@ -1701,7 +1710,10 @@ extern "C" fs_status fs_batch_solve(fs_batch* b, const float* const* d_I0,
       b->warps = warps;
       b->iters = iters;
     }
-    for (int i = 0; i < n; ++i) b->h[i]->has_state = false;
+    for (int i = 0; i < n; ++i) {
+      b->h[i]->has_state = false;
+      constants_stale(b->h[i]);
+    }
     FS_CUDA(cudaGraphLaunch(b->gexec, b->stream));
     FS_CUDA(cudaStreamSynchronize(b->stream));
     if (*b->plan->h_status != 0)
@@ -1749,6 +1761,7 @@ extern "C" fs_status fs_batch_solve(fs_batch* b, const float* const* d_I0,
     b->warps = warps;
     b->iters = iters;
   }
+  for (int i = 0; i < n; ++i) constants_stale(b->h[i]);
   FS_CUDA(cudaGraphLaunch(b->gexec, b->stream));
   for (int i = 0; i < n; ++i) {
     fs_handle* h = b->h[i];
