@@ -51,7 +51,10 @@ typedef enum {
  * "stage" (fs_solve_host's staging planes), "sched" (the accelerated
  * schedule's table), "energy" (fs_energy's accumulators), "planes" (a served
  * rig's image and output planes) -- that device allocation fails without
- * reaching the device, and the call returns FS_ENOMEM. */
+ * reaching the device, and the call returns FS_ENOMEM.  While FS_FAULT_WAIT
+ * is a number of seconds in (0, 3600], handles are created with
+ * fs_persist_stall on and that wait limit (fs_stages.h): the bounded waits of
+ * their solves run out. */
 
 /* Radially symmetric camera models, pixel = c + f * r(theta) * (X, Y)/|(X, Y)|
  * with theta the angle off the optical axis (Sec. III-B allows any model
@@ -210,7 +213,13 @@ fs_status fs_trajectory_field(fs_handle* h, int level, float* d_out);
  * level; else a W x H disparity (px) to warm-start from, in which case only
  * the finest level runs.  warps >= 1 warps of iters >= 1 primal-dual
  * iterations per level.  d_disp (W x H, px along the epipolar curve) and
- * d_depth (W x H, metres along the camera-0 ray) may be NULL to skip. */
+ * d_depth (W x H, metres along the camera-0 ray) may be NULL to skip.
+ * Asynchronous on the handle's stream, except in the persistent schedule.
+ * Large levels (from about 1280 x 1280) run footprints whose copies into
+ * shared memory are waited for with a bound (fs_set_wait_limit, 2 s): should
+ * such a wait run out, the outputs are unspecified, and fs_check_waits
+ * (fs_stages.h), called once the work is done, returns FS_ETIMEOUT.  The same
+ * holds for fs_solve_continue and, for each of its handles, fs_batch_solve. */
 fs_status fs_solve(fs_handle* h, const float* d_I0, const float* d_I1,
                    const float* d_init, int warps, int iters,
                    float* d_disp, float* d_depth);
@@ -232,7 +241,7 @@ fs_status fs_solve_continue(fs_handle* h, const float* d_I0, const float* d_I1, 
 /* (No counterpart in the paper: the end-to-end host entry point.)
  * fs_solve from HOST buffers: copies the inputs to the device, solves,
  * copies the outputs back and synchronises the handle's stream before
- * returning.  Host buffers may be pageable or pinned (pinned is faster). */
+ * returning; FS_ETIMEOUT where fs_check_waits would return it.  Host buffers may be pageable or pinned (pinned is faster). */
 fs_status fs_solve_host(fs_handle* h, const float* h_I0, const float* h_I1,
                         const float* h_init, int warps, int iters,
                         float* h_disp, float* h_depth);
@@ -267,7 +276,8 @@ fs_status fs_batch_create(fs_handle* const* handles, int n, void* cuda_stream,
 /* Arrays of n device pointers, as for fs_solve per pair; d_init may be NULL
  * (all cold starts) or hold NULL entries; d_disp / d_depth entries may be
  * NULL.  warps >= 1, iters >= 1 for every pair.  Asynchronous on the batch
- * stream. */
+ * stream; bounded copy waits as for fs_solve (synchronise the batch stream
+ * before fs_check_waits of a handle, which only waits for the handle's own). */
 fs_status fs_batch_solve(fs_batch* b, const float* const* d_I0, const float* const* d_I1,
                          const float* const* d_init, int warps, int iters,
                          float* const* d_disp, float* const* d_depth);

@@ -114,7 +114,8 @@ fs_status fs_server_submit(fs_server* s, int rig, const float* h_I0, const float
                            float* h_disp, float* h_depth, long long* req_id);
 
 /* Wait up to timeout_s seconds (< 0: no limit) for a request.  On
- * completion returns the request's own status (FS_OK or the error it met),
+ * completion returns the request's own status (FS_OK or the error it met;
+ * FS_ECUDA where a bounded copy wait of its solve ran out, see fs_check_waits),
  * forgets the request, and sets *latency_ms (may be NULL).  FS_ETIMEOUT if
  * it is still pending (it stays known); FS_EINVAL for an unknown id, or
  * while another thread is already waiting for the same request (threads

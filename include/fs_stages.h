@@ -184,8 +184,9 @@ fs_status fs_persist_stall(fs_handle* h, int stall);
  * FS_ETIMEOUT (the state of the levels involved is then unspecified) when a
  * wait ran out since the last check, clearing the record, else FS_OK.
  * fs_solve_host checks by itself when the handle's schedule uses these
- * footprints; fs_solve, fs_solve_continue and fs_batch_solve enqueue work
- * and leave the check to the caller. */
+ * footprints, and the server per request; fs_solve, fs_solve_continue and
+ * fs_batch_solve enqueue work and leave the check to the caller (for a batch,
+ * once its own stream has been synchronised). */
 fs_status fs_check_waits(fs_handle* h);
 
 #ifdef __cplusplus

@@ -262,7 +262,10 @@ class Solver:
         return t.contiguous()
 
     def solve(self, I0, I1, warps, iters, init=None, disp=None, depth=None):
-        """fs_solve on device tensors (H, W); returns (disparity, depth) tensors."""
+        """fs_solve on device tensors (H, W); returns (disparity, depth) tensors.
+        Asynchronous: on large levels check_waits() tells, once the work is
+        done, whether a bounded copy wait ran out (as for solve_continue and
+        Batch.solve; solve_host and the server check by themselves)."""
         torch = self.torch
         I0 = self._dev(I0)
         I1 = self._dev(I1)

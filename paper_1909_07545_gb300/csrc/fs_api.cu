@@ -1202,6 +1202,11 @@ fs_status fs_create(const fs_calib cam[2], const fs_pose* pose, int W, int H, in
   h->H = H;
   h->L = levels;
   h->stream = (cudaStream_t)cuda_stream;
+  const char* wenv = std::getenv("FS_FAULT_WAIT");
+  if (wenv && std::atof(wenv) > 0 && std::atof(wenv) <= 3600) {
+    h->persist_stall = 1;
+    h->wait_ns = (unsigned long long)(std::atof(wenv) * 1e9);
+  }
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -1541,6 +1546,18 @@ static fs_status solve_impl(fs_handle* h, const float* d_I0, const float* d_I1,
   fs_status s = solve_launch(h, d_I0, d_I1, d_init, cont, warps, iters, d_disp, d_depth);
   if (s == FS_OK && h->guard) s = fs_guard_check(h);
   return s;
+}
+
+// For the server: behind a solve of `iters` iterations a warp, on the handle's
+// stream, the record of copy waits to the pinned word *late and cleared (what
+// fs_check_waits reads, without a wait); *late = 0 at once where the handle's
+// schedule makes no such waits.
+fs_status fs_internal_take_waits(fs_handle* h, int iters, int* late) {
+  *late = 0;
+  if (!uses_tma(h, iters)) return FS_OK;
+  FS_CUDA(cudaMemcpyAsync(late, h->pd_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  FS_CUDA(cudaMemsetAsync(h->pd_status, 0, sizeof(int), h->stream));
+  return FS_OK;
 }
 
 extern "C" {
@@ -2151,6 +2168,8 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
   h->prm.pd_schedule = saved_sched;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  // a trial's copy wait that ran out is no later solve's
+  FS_CUDA(cudaMemsetAsync(h->pd_status, 0, sizeof(int), h->stream));
   return st;
 }
 

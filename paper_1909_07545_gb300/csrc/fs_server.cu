@@ -35,6 +35,7 @@ extern fs_status fs_internal_set_error(fs_status s, const char* msg);
 extern fs_status fs_internal_validate(const fs_calib cam[2], const fs_pose* pose, int W, int H,
                                       int levels, const fs_params* prm);
 extern cudaError_t fs_internal_malloc(void** p, size_t bytes, const char* site);
+extern fs_status fs_internal_take_waits(fs_handle* h, int iters, int* late);
 
 namespace {
 
@@ -63,6 +64,7 @@ struct Rig {
   fs_handle* h = nullptr;         // resident state (null: not resident)
   float* planes = nullptr;        // I0, I1, disparity (also the warm start), depth
   cudaStream_t stream = nullptr;
+  int* late = nullptr;            // pinned: a copy wait of the request's solve ran out
   bool has_prev = false;          // planes hold the previous frame's disparity
   bool busy = false;              // a request of this rig is in flight
   unsigned long long last_use = 0;
@@ -122,7 +124,13 @@ void CUDART_CB on_request_done(void* arg) {
     std::lock_guard<std::mutex> g(s->mu);
     r->t_done = t;
     r->done = true;
-    s->rigs[r->rig]->busy = false;
+    Rig* rg = s->rigs[r->rig];
+    if (*rg->late) {                // the outputs and the level state are unspecified
+      r->status = FS_ECUDA;
+      r->msg = "a copy wait of the TMA-staged primal-dual footprints ran out";
+      rg->has_prev = false;         // the rig's next frame starts cold
+    }
+    rg->busy = false;
     --s->inflight;
     ++s->completed;
     if (r->status != FS_OK) ++s->failed;
@@ -162,6 +170,12 @@ void destroy_detached(const Detached& d) {
 // so nothing else touches it).  Returns FS_OK or the error of fs_create /
 // the plane allocation, with *msg set.
 fs_status make_resident(fs_server* s, Rig* rg, std::string* msg) {
+  if (!rg->late && cudaHostAlloc((void**)&rg->late, sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+    cudaGetLastError();
+    rg->late = nullptr;
+    *msg = "status word allocation failed";
+    return FS_ENOMEM;
+  }
   fs_params p = rg->prm;
   p.use_graph = 1;
   fs_status st = fs_create(rg->cam, &rg->pose, rg->W, rg->H, rg->levels, &p, rg->stream, &rg->h);
@@ -213,6 +227,8 @@ fs_status enqueue_request(fs_server* s, Rig* rg, Request* r, bool cold_start, st
     st_solve = fs_solve_continue(rg->h, dI0, dI1, s->cfg.warps, s->cfg.iters, dD, dZ);
   else
     st_solve = fs_solve(rg->h, dI0, dI1, dD, s->cfg.warps, s->cfg.iters, dD, dZ);
+  if (st_solve == FS_OK)
+    st_solve = fs_internal_take_waits(rg->h, cold_start ? s->cfg.cold_iters : s->cfg.iters, rg->late);
   if (st_solve != FS_OK) {
     *msg = fs_last_error();
     return st_solve;
@@ -282,6 +298,7 @@ bool admit_one(fs_server* s, std::unique_lock<std::mutex>& lk) {
     s->peak = std::max(s->peak, s->resident);
     const bool cold_start = need_state || !rg->has_prev;
     if (cold_start) ++s->cold;
+    rg->has_prev = true;                        // unless it fails, here or in on_request_done
     lk.unlock();
     for (const Detached& d : evicted) destroy_detached(d);
     std::string msg;
@@ -290,6 +307,7 @@ bool admit_one(fs_server* s, std::unique_lock<std::mutex>& lk) {
       lk.lock();
       s->resident -= rg->bytes;
       rg->busy = false;
+      rg->has_prev = false;
       --s->inflight;
       fail_request(s, r, st, msg);
       s->cv_done.notify_all();
@@ -303,8 +321,6 @@ bool admit_one(fs_server* s, std::unique_lock<std::mutex>& lk) {
       rg->has_prev = false;
       fail_request(s, r, st, msg);
       s->cv_done.notify_all();
-    } else {
-      rg->has_prev = true;
     }
     return true;
   }
@@ -577,6 +593,7 @@ fs_status fs_server_destroy(fs_server* s) {
   for (Rig* rg : s->rigs) {
     destroy_detached(detach_rig_state(s, rg));
     if (rg->stream) cudaStreamDestroy(rg->stream);
+    if (rg->late) cudaFreeHost(rg->late);
     delete rg;
   }
   for (auto& kv : s->known) delete kv.second;
