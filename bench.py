@@ -77,12 +77,12 @@ def decode_choice(c):
 
 
 def schedule_label(c):
-    """fs_autotune's per-level choice in words (0 = cluster; 1..48 = depth
+    """A level's schedule in words (-1 = automatic; 0 = cluster; 1..48 = depth
     1..8 on each of the six footprints; 49..55 = depth 9..15 on 32x32
     footprints of 1024 threads; 56..63 = depth 1..8 on the TMA-staged
     footprints; 64..71 = depth 1..8 on 64x48 footprints of 768 threads)."""
-    if c == 0:
-        return "cluster"
+    if c <= 0:
+        return "cluster" if c == 0 else "automatic (footprint and depth by level size and iterations)"
     B, v = decode_choice(c)
     return f"blocking x{B} ({FOOTPRINTS[v]})"
 
@@ -483,7 +483,8 @@ def uneven_batch_leg(seed, stream, steps, warmup, storage="f16", per_size=16,
                        lam=p["lam"], huber_eps=p["eps"], use_graph=1, storage=st,
                        pd_schedule=sched)
             if W not in tuned:
-                tuned[W] = x.autotune(p["iters"])
+                x.autotune(p["iters"])
+                tuned[W] = x.schedule()
             else:
                 x.set_schedule(tuned[W])
             sols.append(x)
@@ -718,7 +719,9 @@ def main():
         s = Solver(pair["cam0"], pair["cam1"], pair["R"], pair["t"], W, H, L, stream=stream,
                    lam=pair["lam"], huber_eps=pair["eps"], use_graph=1,
                    block_iters=args.block_iters)
-        tuned = s.autotune(iters) if args.autotune else None
+        # the fastest encoded choices, and the schedule the handle keeps
+        encoded = s.autotune(iters) if args.autotune else None
+        tuned = s.schedule() if args.autotune else None
         # pixels inside each level's FOV mask (the pixels the method moves)
         mask_px = [int((s.read(l, "MASK") > 0.5).sum().item()) for l in range(L)]
         I0 = torch.as_tensor(np.float32(pair["I0"]), device="cuda")
@@ -845,7 +848,9 @@ def main():
         # the paper's own regulariser, TGV-L1 (Eq. 10-11): same frame, FP32
         x = Solver(pair["cam0"], pair["cam1"], pair["R"], pair["t"], W, H, L, stream=stream,
                    lam=pair["lam"], huber_eps=pair["eps"], use_graph=1, regularizer="tgv")
-        tgv_sched = x.autotune(iters) if args.autotune else None
+        if args.autotune:
+            x.autotune(iters)
+        tgv_sched = x.schedule() if args.autotune else None
         ms = timed(lambda: x.solve(I0, I1, warps, iters, disp=disp, depth=depth), vsteps)
         variants["tgv_f32"] = {"value": job_rate(world, 1, ms), "unit": "frames/s",
                                "ms_per_frame": ms,
@@ -855,8 +860,8 @@ def main():
         # work list (footprints and depths from the same tuning)
         x = Solver(pair["cam0"], pair["cam1"], pair["R"], pair["t"], W, H, L, stream=stream,
                    lam=pair["lam"], huber_eps=pair["eps"], use_graph=1, pd_schedule="persistent")
-        if tuned:
-            x.set_schedule(tuned)
+        if encoded:
+            x.set_schedule(encoded)
         ms = timed(lambda: x.solve(I0, I1, warps, iters, disp=disp, depth=depth), vsteps)
         variants["persistent_f32"] = {"value": job_rate(world, 1, ms), "unit": "frames/s",
                                       "ms_per_frame": ms,
@@ -868,7 +873,7 @@ def main():
     # plain FP32 single-pair figure above
     batch1024 = None
     if args.batch > 1:
-        batch1024 = batch_1024_leg(args.seed, stream, tuned, max(3, min(args.steps, 10)),
+        batch1024 = batch_1024_leg(args.seed, stream, encoded, max(3, min(args.steps, 10)),
                                    args.warmup, n=args.batch)
 
     uneven = None
@@ -900,14 +905,8 @@ def main():
     fps = job_rate(world, args.steps, total_ms)
     ms0, n0, px0 = per_level[0]
     launch_s = ms0 / 1000.0 / max(n0, 1)                # mean level-0 launch duration
-    l0_choice = tuned[0] if tuned else None
+    l0_choice = tuned[0] if tuned else -1
     dec = decode_choice(l0_choice)
-    if dec is not None:
-        # the tuner keeps the automatic schedule where that is faster than the
-        # choice it reports: seen by another number of launches
-        n = -(-iters // dec[0])
-        if n0 // max(args.steps, 1) != warps * (n + n % 2):
-            l0_choice, dec = None, None
     peaks, src = measured_peaks()
     peak = float(peaks["hbm_gbs"])
     # Algorithmic bytes of one level-0 launch (the blocked figure of the
@@ -965,7 +964,7 @@ def main():
                      "traffic_frac": traffic / launch_s / 1e9 / peak if traffic else None,
                      "kernel": ("k_pd_tma" if dec is not None and dec[1] == TMA_FOOTPRINT
                                 else "k_pd") + " level 0 (1024x1024), " + (
-                         schedule_label(l0_choice) if l0_choice is not None else "automatic schedule"),
+                         schedule_label(l0_choice)),
                      "launches_per_frame": n0 // max(args.steps, 1),
                      "launch_us": launch_s * 1e6,
                      "algorithmic_bytes_per_launch": bytes_launch,

@@ -118,16 +118,24 @@ fs_status fs_timing_read(fs_handle* h, double* ms, long long* launches,
  * candidates are 0 = a dual and a primal launch per iteration and 8 v + d =
  * temporal-blocking depth d on a 32 x 32 footprint of 256 (v = 0, choices
  * 1..8), 1024 (v = 1, 9..16) or 512 threads (v = 2, 17..24), or a 64 x 32
- * footprint of 512 (v = 3, 25..32) or 1024 threads (v = 4, 33..40).  Each level is timed
- * once more in the automatic schedule, whose footprints and depths go beyond
- * this encoding: where that is faster, the handle keeps it and choice reports
- * the fastest encoded one.  Overwrites the levels' state; synchronises the
+ * footprint of 512 (v = 3, 25..32) or 1024 threads (v = 4, 33..40).  choice is the
+ * fastest of these.  In FP32 storage and outside the persistent schedule each
+ * level is timed once more in the automatic schedule, whose footprints and
+ * depths go beyond this encoding: where that is faster still, the handle keeps
+ * it, and fs_get_schedule says so.  Overwrites the levels' state; synchronises the
  * stream.  All candidates give identical results. */
 fs_status fs_autotune(fs_handle* h, int iters, int* choice);
 
+/* The schedule each level of the handle runs, one entry per level in
+ * fs_autotune's encoding, -1 = the automatic schedule: what fs_autotune,
+ * fs_set_schedule or fs_batch_autotune left (all -1 on a new handle).
+ * fs_set_schedule of it on a handle of the same size and parameters reproduces
+ * the tuning.  FS_EINVAL for a null argument. */
+fs_status fs_get_schedule(const fs_handle* h, int* choice);
+
 /* Set the per-level schedule directly, in fs_autotune's encoding (one entry
- * per level; -1 = the library default for that level), e.g. to reuse a
- * tuning measured earlier.  FS_EINVAL for a value out of range or a cluster
+ * per level; -1 = the automatic schedule for that level), e.g. to reuse a
+ * tuning measured earlier (fs_get_schedule).  FS_EINVAL for a value out of range or a cluster
  * choice (0) on a level that does not fit one cluster. */
 fs_status fs_set_schedule(fs_handle* h, const int* choice);
 

@@ -47,7 +47,8 @@ EXPORTED = ["fs_default_params", "fs_create", "fs_set_pose", "fs_level_size",
             "fs_stage_depth", "fs_timing_enable", "fs_timing_read", "fs_pd_iterate_noalloc",
             "fs_batch_create", "fs_batch_solve", "fs_batch_set_finest_limit",
             "fs_batch_autotune",
-            "fs_batch_destroy", "fs_autotune", "fs_set_schedule", "fs_energy", "fs_state_bytes",
+            "fs_batch_destroy", "fs_autotune", "fs_set_schedule", "fs_get_schedule", "fs_energy",
+            "fs_state_bytes",
             "fs_guard_check", "fs_guard_clobber", "fs_set_wait_limit", "fs_persist_stall",
             "fs_check_waits",
             "fs_server_default_config", "fs_server_create", "fs_server_add_rig",
@@ -146,6 +147,7 @@ def load_library():
         "fs_batch_destroy": [_P],
         "fs_autotune": [_P, i, _P],
         "fs_set_schedule": [_P, _P],
+        "fs_get_schedule": [_P, _P],
         "fs_guard_check": [_P],
         "fs_guard_clobber": [_P, i, ctypes.c_size_t, ctypes.POINTER(i)],
         "fs_set_wait_limit": [_P, d],
@@ -352,16 +354,16 @@ class Solver:
 
     def autotune(self, iters=20):
         """Pick the primal-dual schedule per level by timing (fs_autotune).
-        Returns per level the choice kept, in fs_autotune's encoding
+        Returns per level the fastest choice of fs_autotune's encoding
         (include/fs_stages.h): 0 = the whole-level cluster; 8 v + d =
         temporal-blocking depth d (1..8) on footprint v (0..5: 64x64 of 512
         threads, 32x32 of 256, 64x32 of 256, 64x64 of 1024, 32x32 of 1024,
         32x32 of 512), so 1..48; 49..55 = depth 9..15 on 32x32 of 1024
         threads; 56..63 = depth 1..8 on the TMA-staged 64x64 footprints;
-        64..71 = depth 1..8 on 64x48 of 768 threads.  (Where the automatic
-        schedule is faster than all of them the handle keeps that, and the
-        best of these is returned.)  TGV handles: 0 = a launch per step,
-        8 v + d = depth d on the five TGV footprints."""
+        64..71 = depth 1..8 on 64x48 of 768 threads.  TGV handles: 0 = a
+        launch per step, 8 v + d = depth d on the five TGV footprints.  In FP32
+        storage the handle keeps the automatic schedule on a level where that
+        is faster still; schedule() is what it keeps."""
         out = (ctypes.c_int * 8)()
         _check(self.lib.fs_autotune(self.h, int(iters), out))
         return [out[l] for l in range(self.levels)]
@@ -372,8 +374,16 @@ class Solver:
         _check(self.lib.fs_energy(self.h, int(level), out))
         return tuple(out)
 
+    def schedule(self):
+        """The per-level schedule in use, in autotune()'s encoding (-1 = the
+        automatic one): set_schedule() of it on another handle of this size
+        and these parameters reproduces this one's tuning."""
+        out = (ctypes.c_int * 8)()
+        _check(self.lib.fs_get_schedule(self.h, out))
+        return [out[l] for l in range(self.levels)]
+
     def set_schedule(self, choice):
-        """Set the per-level schedule in autotune()'s encoding (-1 = default)."""
+        """Set the per-level schedule in autotune()'s encoding (-1 = automatic)."""
         arr = (ctypes.c_int * 8)(*([int(c) for c in choice] + [-1] * (8 - len(choice))))
         _check(self.lib.fs_set_schedule(self.h, arr))
 

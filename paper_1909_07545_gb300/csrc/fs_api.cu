@@ -72,7 +72,6 @@ struct HostLevel {
   mutable PdSchedule plan[2];
   mutable int plan_iters[2] = {-1, -1}, plan_nl[2] = {-1, -1};
   bool flipped = false;                     // the two buffer sets have changed places (flip_sets)
-  bool auto_best = false;                   // the tuner found pd_auto's schedule faster still
   LevelView v{};
   // tensor maps of the TMA-staged primal-dual footprints, reading buffer
   // set 0 (primary) and set 1 (alternate); tma_ok = false if the driver
@@ -444,7 +443,7 @@ bool use_cluster(const fs_handle* h, int l) {
   const HostLevel& L = h->lv[l];
   if (L.cluster < 0 || h->prm.pd_schedule != 0 || h->prm.accel_gamma > 0) return false;
   if (h->prm.block_iters <= 0 && L.tuned >= 1) return false;   // tuner chose blocking
-  return L.tuned == 0 && !L.auto_best ? true : h->prm.storage != ST_F32;
+  return L.tuned == 0 || h->prm.storage != ST_F32;
 }
 
 // The temporal-blocking launches of `iters` iterations on level l: the tuned
@@ -456,8 +455,8 @@ PdSchedule pd_plan(const fs_handle* h, int l, int iters, bool odd = false) {
   const HostLevel& L = h->lv[l];
   const int b = std::min(h->prm.block_iters, 8);
   const bool tgv = h->prm.regularizer == FS_REG_TGV;
-  if (tgv && b <= 0 && L.tuned == 0 && !L.auto_best) return PdSchedule{};
-  if (b <= 0 && L.tuned >= 1 && !L.auto_best) {
+  if (tgv && b <= 0 && L.tuned == 0) return PdSchedule{};
+  if (b <= 0 && L.tuned >= 1) {
     const int nl = pd_launch_count(iters, L.tuned);
     return PdSchedule{L.tuned_variant, nl, (iters + nl - 1) / nl, false};
   }
@@ -1819,11 +1818,7 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
   if (choice) *choice = -1;
   const int n = (int)b->h.size();
   // every handle's own coarse choices (to restore when they win)
-  struct Own {
-    int tuned, variant;
-    bool auto_best;
-  };
-  std::vector<std::vector<Own>> own(n);
+  std::vector<std::vector<std::pair<int, int>>> own(n);
   bool any = false;
   for (int i = 0; i < n; ++i) {
     fs_handle* h = b->h[i];
@@ -1832,7 +1827,7 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
     fs_status s;
     if ((s = ensure_schedule(h, iters)) != FS_OK) return s;
     for (int l = 2; l < h->L; ++l) {
-      own[i].push_back({h->lv[l].tuned, h->lv[l].tuned_variant, h->lv[l].auto_best});
+      own[i].push_back({h->lv[l].tuned, h->lv[l].tuned_variant});
       any = true;
     }
   }
@@ -1848,11 +1843,9 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
       for (int l = 2; l < h->L; ++l) {
         HostLevel& L = h->lv[l];
         if (c < 0) {
-          L.tuned = own[i][l - 2].tuned;
-          L.tuned_variant = own[i][l - 2].variant;
-          L.auto_best = own[i][l - 2].auto_best;
+          L.tuned = own[i][l - 2].first;
+          L.tuned_variant = own[i][l - 2].second;
         } else {
-          L.auto_best = false;
           decode_choice(c, false, L.tuned, L.tuned_variant);
         }
       }
@@ -2109,7 +2102,6 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
     HostLevel& L = h->lv[l];
     L.tuned = -1;
     L.tuned_variant = -1;
-    L.auto_best = false;
     float best = 3.4e38f;
     int best_c = -1;
     std::vector<float> timed(kMaxChoice + 1, -1.f);
@@ -2152,16 +2144,19 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
         if (L.tma_ok || !is_tma_choice(cand, false)) try_cand(cand);
     }
     // the automatic schedule, whose footprints and depths go beyond the
-    // encoding: where it is faster still, the handle keeps it and `choice`
-    // reports the best encoded one
-    bool auto_best = false;
-    if (saved_block <= 0 && st == FS_OK) {
-      h->prm.pd_schedule = saved_sched == 0 ? 0 : 1;
+    // encoding: where it is faster still, the handle keeps it
+    // (fs_get_schedule).  Not in 16-bit storage, where the results depend on
+    // the launches, so that `choice` says what the handle runs; nor where the
+    // persistent schedule takes its geometry from the choice.
+    bool keep_auto = false;
+    if (saved_block <= 0 && h->prm.storage == ST_F32 && saved_sched != FS_SCHED_PERSISTENT &&
+        st == FS_OK) {
+      h->prm.pd_schedule = saved_sched;
       L.tuned = L.tuned_variant = -1;
-      auto_best = time_level() < best;
+      keep_auto = time_level() < best;
     }
-    decode_choice(best_c, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
-    L.auto_best = auto_best;
+    if (!keep_auto)
+      decode_choice(best_c, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
     if (choice) choice[l] = best_c;
   }
   h->prm.block_iters = saved_block;
@@ -2217,7 +2212,23 @@ extern "C" fs_status fs_set_schedule(fs_handle* h, const int* choice) {
     int c = choice[l];
     HostLevel& L = h->lv[l];
     decode_choice(c, tgv, L.tuned, L.tuned_variant);
-    L.auto_best = false;
+  }
+  return FS_OK;
+}
+
+extern "C" fs_status fs_get_schedule(const fs_handle* h, int* choice) {
+  fs_status s;
+  if ((s = check_handle(h)) != FS_OK) return s;
+  if (!choice) return fail(FS_EINVAL, "null schedule");
+  const bool tgv = h->prm.regularizer == FS_REG_TGV;
+  for (int l = 0; l < h->L; ++l) {
+    const HostLevel& L = h->lv[l];
+    choice[l] = -1;
+    for (int c = 0; c <= (tgv ? kMaxTgvChoice : kMaxChoice) && choice[l] < 0; ++c) {
+      int depth, variant;
+      decode_choice(c, tgv, depth, variant);
+      if (depth == L.tuned && variant == L.tuned_variant) choice[l] = c;
+    }
   }
   return FS_OK;
 }
