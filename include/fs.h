@@ -300,8 +300,8 @@ fs_status fs_batch_set_finest_limit(fs_batch* b, int k);
  * instead.  Every handle keeps its own schedule for its two finest levels;
  * for its coarser levels (level 2 and up) this tries, besides every
  * handle's own choices, one common schedule for all pairs from a fixed set
- * (fs_autotune encoding 32, 69, 8, 45), timing `iters` primal-dual
- * iterations on every coarse level of every pair with all pairs at once
+ * (fs_autotune encoding 32, 69, 8, 45), timing two warps of `iters`
+ * primal-dual iterations on every coarse level of every pair with all pairs at once
  * on the batch's streams, and keeps the fastest (written into the handles,
  * as fs_set_schedule would).  choice (may be NULL): the common coarse
  * choice kept, or -1 for the handles' own.  Results are unchanged (every

@@ -120,9 +120,9 @@ fs_status fs_timing_read(fs_handle* h, double* ms, long long* launches,
  * 1..8), 1024 (v = 1, 9..16) or 512 threads (v = 2, 17..24), or a 64 x 32
  * footprint of 512 (v = 3, 25..32) or 1024 threads (v = 4, 33..40).  choice is the
  * fastest of these.  In FP32 storage and outside the persistent schedule each
- * level is timed once more in the automatic schedule, whose footprints and
- * depths go beyond this encoding: where that is faster still, the handle keeps
- * it, and fs_get_schedule says so.  Overwrites the levels' state; synchronises the
+ * level's choice is then timed against the automatic schedule, whose footprints
+ * and depths go beyond this encoding, over two warps as a solve runs them:
+ * where the automatic schedule is faster, the handle keeps it, and fs_get_schedule says so.  Overwrites the levels' state; synchronises the
  * stream.  All candidates give identical results. */
 fs_status fs_autotune(fs_handle* h, int iters, int* choice);
 

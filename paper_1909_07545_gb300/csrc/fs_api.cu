@@ -1851,9 +1851,10 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
       }
     }
   };
-  // `iters` iterations on every coarse level of every pair, each pair on its
-  // own lane (coarsest first), all pairs at once: one graph per candidate,
-  // best of three replays after one
+  // the iterations of two warps (in odd numbers of launches, where a solve
+  // takes them) on every coarse level of every pair, each pair on its own lane
+  // (coarsest first), all pairs at once: one graph per candidate, best of three
+  // replays after one
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   FS_CUDA(cudaEventCreate(&e0));
   FS_CUDA(cudaEventCreate(&e1));
@@ -1865,8 +1866,10 @@ extern "C" fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice) {
     cudaError_t e = cudaEventRecord(b->fork, b->origin);
     for (int i = 0; i < n && s == FS_OK && e == cudaSuccess; ++i) {
       e = cudaStreamWaitEvent(b->lanes[i], b->fork, 0);
-      for (int l = b->h[i]->L - 1; l >= 2 && s == FS_OK && e == cudaSuccess; --l)
-        s = run_pd(b->h[i], l, iters, b->lanes[i]);
+      SetsGuard guard{b->h[i]};
+      for (int l = b->h[i]->L - 1; l >= 2; --l)
+        for (int w = 0; w < 2 && s == FS_OK && e == cudaSuccess; ++w)
+          s = run_pd(b->h[i], l, iters, b->lanes[i], false, w, odd_launches(b->h[i], w, 2));
       if (s == FS_OK && e == cudaSuccess) e = cudaEventRecord(b->joins[i], b->lanes[i]);
       if (s == FS_OK && e == cudaSuccess) e = cudaStreamWaitEvent(b->origin, b->joins[i], 0);
     }
@@ -2105,12 +2108,27 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
     float best = 3.4e38f;
     int best_c = -1;
     std::vector<float> timed(kMaxChoice + 1, -1.f);
-    // best of 3 timed runs of the level's schedule as it stands, after a warm-up
-    auto time_level = [&]() {
+    // best of 3 timed runs, after a warm-up, of the level's schedule as it
+    // stands: one warp's iterations alone, or two warps as enqueue_solve issues
+    // them (odd numbers of launches, chains)
+    auto two_warps = [&]() -> fs_status {
+      SetsGuard guard{h};
+      fs_status r = run_stage(h, l, FS_STAGE_WARP, 0, h->stream);
+      for (int w = 0; w < 2 && r == FS_OK; ++w) {
+        const bool odd = odd_launches(h, w, 2);
+        r = run_pd(h, l, iters, h->stream, true, w, odd);
+        if (r == FS_OK && w == 0)
+          r = run_stage(h, l, FS_STAGE_CLIP_WARP, 0, h->stream, short_chain(h, l, iters, odd));
+      }
+      return r;
+    };
+    auto time_level = [&](bool warps) {
       float t = 3.4e38f;
       for (int rep = 0; rep < 4 && st == FS_OK; ++rep) {
         cudaError_t e = cudaEventRecord(e0, h->stream);
-        if (e == cudaSuccess && (st = run_pd(h, l, iters, h->stream)) != FS_OK) break;
+        if (e == cudaSuccess &&
+            (st = warps ? two_warps() : run_pd(h, l, iters, h->stream)) != FS_OK)
+          break;
         if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;
@@ -2126,7 +2144,7 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
       h->prm.pd_schedule = cand == 0 ? 0 : 1;
       h->prm.block_iters = saved_block;
       decode_choice(cand, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
-      const float t = time_level();
+      const float t = time_level(false);
       timed[cand] = t;
       if (st == FS_OK && t < best) { best = t; best_c = cand; }
     };
@@ -2144,16 +2162,20 @@ extern "C" fs_status fs_autotune(fs_handle* h, int iters, int* choice) {
         if (L.tma_ok || !is_tma_choice(cand, false)) try_cand(cand);
     }
     // the automatic schedule, whose footprints and depths go beyond the
-    // encoding: where it is faster still, the handle keeps it
-    // (fs_get_schedule).  Not in 16-bit storage, where the results depend on
+    // encoding and which a solve runs in odd numbers of launches too: where it
+    // is faster than the best choice, both as a solve runs them, the handle
+    // keeps it (fs_get_schedule).  Not in 16-bit storage, where the results depend on
     // the launches, so that `choice` says what the handle runs; nor where the
     // persistent schedule takes its geometry from the choice.
     bool keep_auto = false;
     if (saved_block <= 0 && h->prm.storage == ST_F32 && saved_sched != FS_SCHED_PERSISTENT &&
         st == FS_OK) {
+      h->prm.pd_schedule = best_c == 0 ? 0 : 1;
+      decode_choice(best_c, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);
+      const float t = time_level(true);
       h->prm.pd_schedule = saved_sched;
       L.tuned = L.tuned_variant = -1;
-      keep_auto = time_level() < best;
+      keep_auto = time_level(true) < t;
     }
     if (!keep_auto)
       decode_choice(best_c, h->prm.regularizer == FS_REG_TGV, L.tuned, L.tuned_variant);

@@ -54,3 +54,29 @@ def test_every_choice_reads_back(regularizer, last):
         s.set_schedule([c])
         assert s.schedule() == [c]
     s.close()
+
+
+def test_a_tuned_handle_is_no_slower_than_an_untuned_one():
+    # the tuner has to time what a solve runs: odd numbers of launches among
+    # it, which the automatic schedule of this workload is 3 % faster with
+    import torch
+    p = f32pair(synth.plain_small(0))
+    ims = [torch.as_tensor(p[k], dtype=torch.float32, device="cuda") for k in ("I0", "I1")]
+    out = torch.empty(2, *ims[0].shape, device="cuda")
+    tuned, plain = make_solver(p, use_graph=1), make_solver(p, use_graph=1)
+    tuned.autotune(50)
+
+    def us(s, n=8):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        for _ in range(n):
+            s.solve(*ims, 5, 50, disp=out[0], depth=out[1])
+        ev[1].record()
+        torch.cuda.synchronize()
+        return ev[0].elapsed_time(ev[1]) * 1000 / n
+    us(tuned), us(plain)
+    runs = [(us(tuned), us(plain)) for _ in range(12)]
+    a, b = (min(r) for r in zip(*runs))
+    assert a <= 1.02 * b, (a, b)
+    tuned.close()
+    plain.close()
