@@ -307,7 +307,8 @@ fs_status fs_batch_set_finest_limit(fs_batch* b, int k);
  * choice kept, or -1 for the handles' own.  Results are unchanged (every
  * schedule gives the same bits).  Overwrites the coarse levels' state and
  * synchronises the batch stream; FS_EINVAL for TGV handles or iters < 1.
- * A batch graph is recaptured after any schedule change of its handles. */
+ * A batch graph is recaptured after any schedule or pose change of its
+ * handles. */
 fs_status fs_batch_autotune(fs_batch* b, int iters, int* choice);
 
 /* Free the batch (its streams, events and graph; not the handles). */

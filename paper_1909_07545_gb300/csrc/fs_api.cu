@@ -297,7 +297,8 @@ struct fs_handle {
   unsigned long long wait_ns = 2000000000ull;
   int persist_stall = 0;
   // bumped whenever a launch argument a captured graph holds changes (the
-  // schedule, the wait bound, the stall aid): batches key their graphs on it
+  // pose's depth constants, the schedule, the wait bound, the stall aid):
+  // batches key their graphs on it
   unsigned sched_gen = 0;
   // set to FS_ETIMEOUT by a TMA-staged primal-dual launch whose copy wait
   // ran out (in the arena; read and cleared by fs_check_waits)
@@ -1389,6 +1390,7 @@ fs_status fs_set_pose(fs_handle* h, const fs_pose* pose) {
     cudaGraphExecDestroy(h->gexec);
     h->gexec = nullptr;
   }
+  ++h->sched_gen;  // and so did a batch's
   return FS_OK;
 }
 
