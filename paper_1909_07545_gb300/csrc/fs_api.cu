@@ -297,8 +297,8 @@ struct fs_handle {
   unsigned long long wait_ns = 2000000000ull;
   int persist_stall = 0;
   // bumped whenever a launch argument a captured graph holds changes (the
-  // pose's depth constants, the schedule, the wait bound, the stall aid):
-  // batches key their graphs on it
+  // pose's depth constants, the schedule, the wait bound, the stall aid, the
+  // timing events): batches key their graphs on it
   unsigned sched_gen = 0;
   // set to FS_ETIMEOUT by a TMA-staged primal-dual launch whose copy wait
   // ran out (in the arena; read and cleared by fs_check_waits)
@@ -2051,9 +2051,10 @@ extern "C" fs_status fs_stage_prerotate(fs_handle* h, const float* d_I1) {
 extern "C" fs_status fs_timing_enable(fs_handle* h, int enable) {
   fs_status s;
   if ((s = check_handle(h)) != FS_OK) return s;
-  if ((enable != 0) != (h->timing != 0) && h->gexec) {  // captured graph has / lacks the events
-    cudaGraphExecDestroy(h->gexec);
+  if ((enable != 0) != (h->timing != 0)) {  // captured graphs have / lack the events
+    if (h->gexec) cudaGraphExecDestroy(h->gexec);
     h->gexec = nullptr;
+    ++h->sched_gen;
   }
   h->timing = enable != 0;
   h->ev_pending = false;
