@@ -177,7 +177,7 @@ fs_status fs_set_wait_limit(fs_handle* h, double seconds);
  * the finest level of this handle's persistent solves wait for a counter
  * that nothing advances, so that wait runs out, and makes the first launch
  * of every level that runs the TMA-staged footprints (below) wait
- * on a barrier that nothing completes; stall = 0 restores the schedule.  A
+ * for an arrival that does not come; stall = 0 restores the schedule.  A
  * batch stalls when any of its handles does.  Both this call and
  * fs_set_wait_limit drop the handle's captured graph (the bound and the
  * stall are launch arguments); a batch's graph keeps the values it was

@@ -90,6 +90,10 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, unsigned bytes) {
                : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, unsigned parity) {
   unsigned done;
   asm volatile(
@@ -144,7 +148,7 @@ __device__ __forceinline__ float sval(const unsigned char* plane, int k) {
 // set `in` and written to `out`.  chained (pd_tile): PD_CHAINED requests the
 // first footprint's constants before the wait for the preceding launch and
 // its state after, PD_CHAIN_START waits first.  stall: testing aid, the
-// first wait is on a barrier that nothing completes.
+// first wait's barrier expects an arrival that only comes when it is given up.
 //
 // Bound by the iterations, 1450-1700 clock cycles each, and by what lies
 // between two footprints: 3800 cycles, the 1400 shared-memory wavefronts of
@@ -171,7 +175,6 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   float(*s_t1)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_t1);
   float(*s_t2)[kFW] = reinterpret_cast<float(*)[kFW]>(smem + Lay::x_t2);
   const uint32_t bar = smem_addr(smem + Lay::bar);
-  const uint32_t wait_bar = smem_addr(smem + Lay::bar + (stall ? 32 : 0));
   volatile int* s_late = reinterpret_cast<volatile int*>(smem + Lay::bar + 16);
 
   // footprint t's place; by: a row at or before it (only ever moves down)
@@ -191,8 +194,7 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   if (chained) cudaTriggerProgrammaticLaunchCompletion();
   int tile = blockIdx.x, by = 0, bx = tile < ntiles ? column(tile, by) : 0;
   if (leader) {
-    mbar_init(bar, 1);
-    if (stall) mbar_init(wait_bar, 1);
+    mbar_init(bar, stall ? 2 : 1);
     *s_late = 0;
     if (tile < ntiles) mbar_expect_tx(bar, Lay::tx);
   }
@@ -206,9 +208,9 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
   unsigned parity = 0;
   while (tile < ntiles) {
     const unsigned long long t0 = global_ns();
-    while (!mbar_try_wait(wait_bar, parity)) {
+    while (!mbar_try_wait(bar, parity)) {
       if (global_ns() - t0 > wait_ns) {
-        *s_late = 1;
+        *s_late = 1 + (int)parity;
         break;
       }
     }
@@ -246,18 +248,7 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
     // the level with all three mask bits set (outside it the mask reads 0).
     // (s_ub: the last footprint's iterations ended with a barrier.)
     const bool full = __syncthreads_and(mb == 07777u);
-    if (*s_late) {
-      // the footprint's copies may still be under way (the limit can be as
-      // short as a caller likes), and the shared memory they write is another
-      // CTA's once this one has left: one thread stays for them
-      if (leader) {
-        atomicCAS(status, 0, (int)FS_ETIMEOUT);
-        const unsigned long long t1 = global_ns();
-        while (!mbar_try_wait(bar, parity ^ 1u) && global_ns() - t1 <= kDrainNs) {
-        }
-      }
-      return;
-    }
+    if (*s_late) break;
     if (n_iters == 0) __syncthreads();   // s_late and s_ub as if iterations followed
     const int next = tile + (int)gridDim.x;
     int nby = by;
@@ -295,6 +286,21 @@ k_pd_tma(LevelView L, PDState in, PDState out, PDParams pp, int B, int n_iters, 
     tile = next;
     bx = nbx;
     by = nby;
+  }
+
+  if (*s_late) {
+    // the footprint's copies may still be under way (the limit can be as short
+    // as a caller likes), and the shared memory they write is another CTA's
+    // once this one has left: one thread stays for them
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+      atomicCAS(status, 0, (int)FS_ETIMEOUT);
+      const uint32_t b = smem_addr(smem + Lay::bar);
+      if (stall) mbar_arrive(b);
+      const unsigned long long t1 = global_ns();
+      while (!mbar_try_wait(b, (unsigned)(*s_late - 1)) && global_ns() - t1 <= kDrainNs) {
+      }
+    }
+    return;
   }
 
   // the first launch of a warp: all its iterations on the footprints left out
