@@ -215,7 +215,7 @@ fs_status fs_trajectory_field(fs_handle* h, int level, float* d_out);
  * iterations per level.  d_disp (W x H, px along the epipolar curve) and
  * d_depth (W x H, metres along the camera-0 ray) may be NULL to skip.
  * Asynchronous on the handle's stream, except in the persistent schedule.
- * Large levels (from about 1280 x 1280) run footprints whose copies into
+ * Large levels (from about 1100 x 1100) run footprints whose copies into
  * shared memory are waited for with a bound (fs_set_wait_limit, 2 s): should
  * such a wait run out, the outputs are unspecified, and fs_check_waits
  * (fs_stages.h), called once the work is done, returns FS_ETIMEOUT.  The same

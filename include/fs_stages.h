@@ -180,15 +180,16 @@ fs_status fs_set_wait_limit(fs_handle* h, double seconds);
  * for an arrival that does not come; stall = 0 restores the schedule.  A
  * batch stalls when any of its handles does.  Both this call and
  * fs_set_wait_limit drop the handle's captured graph (the bound and the
- * stall are launch arguments); a batch's graph keeps the values it was
- * captured with. */
+ * stall are launch arguments), and a batch captures its own again at its next
+ * solve. */
 fs_status fs_persist_stall(fs_handle* h, int stall);
 
 /* The TMA-staged primal-dual footprints (fs_autotune choices 56..63, and the
- * automatic schedule's choice on the largest levels): each launch's CTAs wait on a shared-memory barrier for the copies of every
- * footprint, bounded like the persistent schedule (fs_set_wait_limit).  A
- * wait that runs out makes its CTA return and records FS_ETIMEOUT in the
- * handle.  fs_check_waits synchronises the handle's stream and returns
+ * automatic schedule's choice on the largest levels): each launch's CTAs wait
+ * on a shared-memory barrier for the copies of every footprint, bounded like
+ * the persistent schedule (fs_set_wait_limit).  A wait that runs out makes its
+ * CTA record FS_ETIMEOUT in the handle and return, once its copies have landed
+ * (or two seconds later).  fs_check_waits synchronises the handle's stream and returns
  * FS_ETIMEOUT (the state of the levels involved is then unspecified) when a
  * wait ran out since the last check, clearing the record, else FS_OK.
  * fs_solve_host checks by itself when the handle's schedule uses these

@@ -447,7 +447,7 @@ constexpr int kBlkX = 32, kBlkY = 8;     // the CTAs of the per-pixel kernels
 // sooner than an ordinary one; so what the launch before wrote besides images
 // is read through L2: 128 x 128 126.4 -> 120.8 us.
 // The step sizes need the tensor at the left and the upper pixel too: a CTA
-// evaluates each once and shares it (640 x 480 frame 302.6 -> 301.0 us, 1024 x
+// evaluates each once and shares it (640 x 640 frame 302.6 -> 301.0 us, 1024 x
 // 1024 6980 -> 6961).
 template <int S, int MODE, bool TGV>
 __global__ void k_level_start(LevelView C, LevelView L, float beta, float eta, int precond,

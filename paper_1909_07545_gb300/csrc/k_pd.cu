@@ -266,9 +266,22 @@ int pd_launch_count(int iters, int depth) {
 //   1024 x 1024  41.9 / 392           47.5 / 434
 //   2048 x 2048 (50 iterations)  816          1034
 // The TMA-staged footprints' third figure is a launch's own time; they win
-// from where an SM has some six footprints: 100 iterations of 2048 x 2048
-// with a 180-degree FOV 1220 us against 1410-1600 (64 x 32, two per SM), a
-// frame 19.6 ms against 23.7; 1024 x 1024 keeps 64 x 32.
+// from where an SM has some three or four footprints, and by more the larger the
+// level: a frame of 2048 x 2048 19.6 ms against 23.7.  The rule takes them from
+// between 1024 x 1024, which keeps 64 x 32, and 1152 x 1152, later for few
+// iterations.  us per 20 / 100 iterations, what it picks against the best it
+// picks without them, with the FOV of a 180-degree lens over the level's width:
+//   1088 x 1088    89 / 404   against    89 / 417
+//   1152 x 1152    98 / 454             109 / 477
+//   1280 x 1280   120 / 528             120 / 566
+//   1536 x 1536   200 / 732             200 / 913
+//   1792 x 1792   217 / 973             262 / 1260
+//   2048 x 2048   258 / 1235            326 / 1590
+// and with the FOV over the whole level:
+//   1024 x 1024    83 / 397   against    82 / 397
+//   1152 x 1152   110 / 488             110 / 550
+//   1536 x 1536   199 / 829             199 / 1065
+//   2048 x 2048   295 / 1453            394 / 1942
 // Where it saves waves, the footprints outside the FOV are left out: a 2048 x
 // 2048 frame under a 180-degree lens takes 24.0 ms against 27.9.  (With a
 // single wave the test only costs, up to 4 % of a 256 x 256 frame.)

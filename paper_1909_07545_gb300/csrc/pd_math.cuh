@@ -78,7 +78,7 @@ __device__ __forceinline__ void px_zero(PxConst& c) {
 // min(1, 1 / sqrt(n2)) for n2 >= 0 (or NaN).  The .ftz form of the
 // approximate reciprocal square root needs no scaling steps for subnormal
 // inputs; it gives the bits of rsqrtf on normal inputs, and on subnormal
-// ones both are above 1 (checked over all 2^31 non-negative floats).  It
+// ones both are above 1 (tests/ball_scale_check.cu: all 2^31 non-negative floats).  It
 // takes 4-5 % off an iteration: 100 iterations at 1024 x 1024 (64 x 64
 // footprints of 1024 threads, depth 7) went from 438 to 419 us.
 __device__ __forceinline__ float ball_scale(float n2) {
